@@ -423,8 +423,13 @@ cudaError_t enq_omp(dl_ctx* c, const float* Y, int64_t m, const float* D, int s)
   e = cudaMemsetAsync(c->rs_count, 0, sizeof(int), c->st);
   if (e != cudaSuccess) return e;
   const bool tm = c->cfg_omp_tm && !has_prop(c) && dlk::omp_tm_supported(c->n, s);
-  c->last_omp = tm ? 1 : 0;
-  if (tm)
+  const bool roll = c->cfg_omp_tm && dlk::omp_roll_supported(c->n, s);
+  c->last_omp = tm || roll ? 1 : 0;
+  if (roll)
+    e = dlk::omp_roll(c->A0, c->lda, c->G, c->n, Y, c->p, m, s, c->sidx, c->sval, c->scnt,
+                      has_prop(c) ? c->rr_ref : nullptr, c->err, c->rs_list, c->rs_count,
+                      (int)c->m_max, lp_ok(c) ? 0.f : dlk::kGapTol, c->st);
+  else if (tm)
     e = dlk::omp_batch_tm(c->cfg_omp_tm, c->A0, c->a0_bf16, c->lda, c->G, c->n, Y, c->p, m, s, c->sidx, c->sval,
                           c->scnt, c->err, c->rs_list, c->rs_count, (int)c->m_max, c->st);
   else
@@ -617,6 +622,7 @@ cudaError_t enq_omp_staged(dl_ctx* c, const float* hostY, const float* dY, int64
     if ((e = cudaEventRecord(c->ev_chunk[q], c->st2)) != cudaSuccess) return e;
   }
   mark(c, 2);
+  const bool roll = c->cfg_omp_tm && dlk::omp_roll_supported(c->n, s);
   bool first = true;
   for (int q = 0; q < dl_ctx::kChunks; ++q) {
     const int64_t off = offs[q], mk = offs[q + 1] - offs[q];
@@ -630,7 +636,11 @@ cudaError_t enq_omp_staged(dl_ctx* c, const float* hostY, const float* dY, int64
     if (e != cudaSuccess) return e;
     first = false;
     if ((e = cudaMemsetAsync(c->rs_count, 0, sizeof(int), c->st)) != cudaSuccess) return e;
-    if (c->cfg_omp_tm && dlk::omp_tm_supported(c->n, s))
+    if (roll)
+      e = dlk::omp_roll(Aq, c->lda, c->G, c->n, Yq, c->p, mk, s, c->sidx + off * s,
+                        c->sval + off * s, c->scnt + off, nullptr, c->err, c->rs_list, c->rs_count,
+                        (int)c->m_max, dlk::kGapTol, c->st);
+    else if (c->cfg_omp_tm && dlk::omp_tm_supported(c->n, s))
       e = dlk::omp_batch_tm(c->cfg_omp_tm, Aq, false, c->lda, c->G, c->n, Yq, c->p, mk, s, c->sidx + off * s,
                             c->sval + off * s, c->scnt + off, c->err, c->rs_list, c->rs_count,
                             (int)c->m_max, c->st);
@@ -646,7 +656,7 @@ cudaError_t enq_omp_staged(dl_ctx* c, const float* hostY, const float* dY, int64
     k += 3;
   }
   mark(c, 3);
-  c->last_omp = c->cfg_omp_tm && dlk::omp_tm_supported(c->n, s) ? 1 : 0;
+  c->last_omp = c->cfg_omp_tm && (roll || dlk::omp_tm_supported(c->n, s)) ? 1 : 0;
   *kernels = k;
   return cudaSuccess;
 }

@@ -99,6 +99,14 @@ cudaError_t omp_batch_tm(int q, const void* A0, bool a0_bf16, int64_t lda, const
                          int32_t* cnt, int* err, int* rs_list, int* rs_count, int rs_cap,
                          cudaStream_t st);
 
+// The arithmetic of omp_batch with rolled loops and the vectors in TMEM and shared
+// memory (k_omp_roll.cu); supported means that it is also the faster one.
+bool omp_roll_supported(int n, int s);
+cudaError_t omp_roll(const float* A0, int64_t lda, const float* G, int n, const float* Y, int p,
+                     int64_t m, int s, int32_t* idx, float* val, int32_t* cnt, float* ores,
+                     int* err, int* rs_list, int* rs_count, int rs_cap, float gap_tol,
+                     cudaStream_t st);
+
 // ---- whole DL iterations of small problems, one CTA per problem (k_small.cu) ----
 // Problems with p <= 32, n <= 64, s <= 8 and group size n: a batch runs all its
 // problems' iterations in one launch.
