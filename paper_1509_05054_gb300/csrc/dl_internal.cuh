@@ -169,7 +169,6 @@ cudaError_t topk_abs(const float* A, int64_t lda, int64_t m, int n, int K, int32
 // the atoms within their error bound), overwriting their slots.  G: the FP32 Gram matrix;
 // A0 (row i = FP32 D^T y_i, stride lda) or null to take D^T y here.  p <= 128, s <= 16.
 constexpr int DL_RESOLVE_SMAX = 16;
-constexpr int DL_RESOLVE_WARPS = 608;  // CTAs of one warp
 cudaError_t omp_resolve64(const float* Y, int p, const float* D, const float* G, const float* A0,
                           int64_t lda, int n, int s, const int* list, const int* count, int cap,
                           int32_t* idx, float* val, int32_t* cnt, cudaStream_t st);

@@ -1,5 +1,5 @@
-"""The rolled Batch-OMP kernel (long supports, wide dictionaries) at the edges of
-its shapes.
+"""The rolled Batch-OMP kernel (long supports, wide dictionaries) and the FP64
+re-solve at the edges of their shapes.
 
 The rolled kernel does the arithmetic of the warp-per-signal kernel operation
 by operation, so the two must agree bit for bit (no tolerance): a context made
@@ -13,7 +13,10 @@ ones (residual stop) and, through a duplicated atom, dependent pivots.
 import numpy as np
 import pytest
 
+import oracle
 from paper_1509_05054_gb300 import synth
+
+from _common import csc_to_slots
 
 pytestmark = pytest.mark.gpu
 
@@ -65,3 +68,24 @@ def test_rolled_kernel_matches_warp_kernel_bit_for_bit(dl, monkeypatch, p, n, s,
     assert res == res0
     for a, b in zip(rolled, warp):
         np.testing.assert_array_equal(a, b)
+
+
+@pytest.mark.parametrize("p", [3, 33, 100, 128])
+def test_resolve_matches_oracle_on_near_dependent_pairs(dl, p):
+    """Atoms e_{p-1} and ~ e_{p-1} + 5e-4 e_{p-2}: an FP32 pivot of 2.5e-7, listed for the FP64
+    re-solve, which finds both (coefficients to FP32 rounding of values up to 2e4: rtol 1e-5)."""
+    E = np.eye(p)
+    b = E[p - 1] + 5e-4 * E[p - 2]
+    D = np.vstack([E[:p - 2], E[p - 1], b / np.linalg.norm(b)]).astype(np.float32)
+    s, m = min(3, p), 50
+    g = np.random.default_rng(5)
+    Y = np.zeros((m, p), np.float32)
+    Y[:, p - 1], Y[:, p - 2] = 2.0, 10.0
+    Y[:, 0] += (g.standard_normal(m) * 0.5).astype(np.float32) if p > 3 else 0.0
+    (cp, ri, v), _, nres = _code(dl, Y, D, s)
+    idx, val, cnt = csc_to_slots(cp, ri, v, s)
+    idx_o, val_o, cnt_o = oracle.omp(Y.astype(np.float64), D.astype(np.float64), s)
+    assert nres == m
+    np.testing.assert_array_equal(cnt, cnt_o)
+    np.testing.assert_array_equal(idx, idx_o)
+    np.testing.assert_allclose(val, val_o, rtol=1e-5, atol=1e-6)
