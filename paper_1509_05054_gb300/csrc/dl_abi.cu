@@ -23,23 +23,27 @@ struct dl_proposer {
   cudaStream_t st = nullptr;
   float* w[6] = {};        // W1 (hidden x pk), b1, W2 (hidden x hidden), b2, W3 (n x hidden), b3
   float* g[6] = {};        // gradients of the last training step
-  float* am[6] = {};       // Adam first moments
-  float* av[6] = {};       // Adam second moments
   int64_t wlen[6] = {};
   void* wb[3] = {};        // BF16 copies of W1, W2, W3
-  void* wt[2] = {};        // BF16 transposes of W2 (hidden x hidden) and W3 (hidden x n)
+  // w, g and wb point into one array each (the same offsets in all; wpad values),
+  // beside the Adam moments, so that one launch updates or clears all of them
+  int64_t wpad = 0;
+  float* wall = nullptr;
+  float* gall = nullptr;
+  float* am = nullptr;     // Adam first moments
+  float* av = nullptr;     // Adam second moments
+  void* wball = nullptr;
   // activations (bmax rows)
   void* X = nullptr;       // BF16 bmax x pk
   float* A1 = nullptr;     // FP32 pre-activations (training)
   float* A2 = nullptr;
   void* H1 = nullptr;      // BF16 activations
   void* H2 = nullptr;
-  float* Z = nullptr;      // FP32 logits (training)
+  float* Z = nullptr;      // FP32 logits (dl_proposer_forward)
   void* Zb = nullptr;      // BF16 logits (inference)
   int32_t* sup = nullptr;  // gathered supports of the batch (bmax x 16)
   // backward scratch (BF16)
-  void *dZ = nullptr, *dZt = nullptr, *H2t = nullptr, *dA2 = nullptr, *dA2t = nullptr, *H1t = nullptr,
-       *dA1 = nullptr, *dA1t = nullptr, *Xt = nullptr;
+  void *dZ = nullptr, *dA2 = nullptr, *dA1 = nullptr;
   double* loss = nullptr;
   int* err = nullptr;
   int step = 0;
@@ -1648,45 +1652,41 @@ constexpr int kPropMaxS = 16;  // support slots gathered per training row
 void free_proposer(dl_proposer* P) {
   if (!P) return;
   DevGuard g(P->dev);
-  for (int k = 0; k < 6; ++k)
-    for (void* q : {(void*)P->w[k], (void*)P->g[k], (void*)P->am[k], (void*)P->av[k]})
-      if (q) cudaFree(q);
-  for (void* q : {P->wb[0], P->wb[1], P->wb[2], P->wt[0], P->wt[1], P->X, (void*)P->A1,
-                  (void*)P->A2, P->H1, P->H2, (void*)P->Z, P->Zb, (void*)P->sup, P->dZ, P->dZt,
-                  P->H2t, P->dA2, P->dA2t, P->H1t, P->dA1, P->dA1t, P->Xt, (void*)P->loss,
-                  (void*)P->err})
+  for (void* q : {(void*)P->wall, (void*)P->gall, (void*)P->am, (void*)P->av, P->wball, P->X,
+                  (void*)P->A1, (void*)P->A2, P->H1, P->H2, (void*)P->Z, P->Zb, (void*)P->sup, P->dZ,
+                  P->dA2, P->dA1, (void*)P->loss, (void*)P->err})
     if (q) cudaFree(q);
   delete P;
 }
 
 int64_t proposer_chunks(dl_proposer* P, int64_t m) { return P ? (m + P->ichunk - 1) / P->ichunk : 0; }
 
-// rows of Y (FP32, p wide; selected by idx when given) -> BF16 rows pk wide, and
-// their support slots (-1 padded to kPropMaxS) when sup is given.
-__global__ void gather_rows_kernel(const float* __restrict__ Y, int p, int pk,
-                                   const int64_t* __restrict__ idx, int64_t B,
-                                   const int32_t* __restrict__ sup_in, int s,
-                                   __nv_bfloat16* __restrict__ X, int32_t* __restrict__ sup_out) {
-  const int64_t e = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
-  if (e >= B * pk) return;
-  const int64_t b = e / pk;
-  const int c = (int)(e - b * pk);
-  const int64_t r = idx ? idx[b] : b;
-  X[e] = __float2bfloat16_rn(c < p ? Y[r * p + c] : 0.f);
-  if (sup_in && c < kPropMaxS) sup_out[b * kPropMaxS + c] = c < s ? sup_in[r * s + c] : -1;
+// The two hidden layers of B rows X (BF16, pk wide); training keeps the FP32 pre-activations.
+cudaError_t enq_hidden(dl_proposer* P, const void* X, int64_t B, bool train) {
+  const int h = P->hidden;
+  dlk::MlpEpi e1{}, e2{};
+  e1.bias = P->w[1];
+  e1.out_f32 = train ? P->A1 : nullptr;
+  e1.out_bf16 = (__nv_bfloat16*)P->H1;
+  e2.bias = P->w[3];
+  e2.out_f32 = train ? P->A2 : nullptr;
+  e2.out_bf16 = (__nv_bfloat16*)P->H2;
+  e1.ldc = e2.ldc = h;
+  cudaError_t e = dlk::mlp_forward(X, B, P->wb[0], h, P->pk, dlk::MLP_EPI_GELU_FWD, e1, P->err, P->st);
+  if (e != cudaSuccess) return e;
+  return dlk::mlp_forward(P->H1, B, P->wb[1], h, h, dlk::MLP_EPI_GELU_FWD, e2, P->err, P->st);
 }
 
-cudaError_t enq_forward_chunk(dl_proposer* P, const void* X, int64_t B, bool train) {
-  const int h = P->hidden;
-  cudaError_t e = dlk::mlp_gemm(X, B, P->wb[0], h, P->pk, dlk::MLP_EPI_GELU_FWD, P->w[1], nullptr, 0,
-                                train ? P->A1 : nullptr, P->H1, h, P->err, P->st);
+// Logits of B rows, as FP32 and/or BF16.
+cudaError_t enq_logits(dl_proposer* P, const void* X, int64_t B, float* z, void* zb) {
+  cudaError_t e = enq_hidden(P, X, B, false);
   if (e != cudaSuccess) return e;
-  e = dlk::mlp_gemm(P->H1, B, P->wb[1], h, h, dlk::MLP_EPI_GELU_FWD, P->w[3], nullptr, 0,
-                    train ? P->A2 : nullptr, P->H2, h, P->err, P->st);
-  if (e != cudaSuccess) return e;
-  return dlk::mlp_gemm(P->H2, B, P->wb[2], P->n, h, train ? dlk::MLP_EPI_F32 : dlk::MLP_EPI_BF16,
-                       P->w[5], nullptr, 0, train ? P->Z : nullptr, train ? nullptr : P->Zb, P->n,
-                       P->err, P->st);
+  dlk::MlpEpi epi{};
+  epi.bias = P->w[5];
+  epi.out_f32 = z;
+  epi.out_bf16 = (__nv_bfloat16*)zb;
+  epi.ldc = P->n;
+  return dlk::mlp_forward(P->H2, B, P->wb[2], P->n, P->hidden, dlk::MLP_EPI_LOGITS, epi, P->err, P->st);
 }
 
 // Logits/top-K of m signals already converted to BF16 rows (pk wide), in chunks
@@ -1697,55 +1697,40 @@ cudaError_t enq_proposer_forward(dl_proposer* P, const void* Xbf, int64_t m, int
   for (int64_t r0 = 0; r0 < m; r0 += P->ichunk) {
     const int64_t B = m - r0 < P->ichunk ? m - r0 : P->ichunk;
     const void* X = (const __nv_bfloat16*)Xbf + r0 * P->pk;
-    cudaError_t e = enq_forward_chunk(P, X, B, false);
+    cudaError_t e = enq_logits(P, X, B, nullptr, P->Zb);
     if (e != cudaSuccess) return e;
     if ((e = dlk::mlp_topk(P->Zb, B, P->n, K, cand + r0 * K, st)) != cudaSuccess) return e;
   }
   return cudaSuccess;
 }
 
-// One training step on B gathered rows already in P->X / P->sup.
+// One training step on B gathered rows already in P->X / P->sup, gradients cleared.
 cudaError_t enq_train_step(dl_proposer* P, int64_t B, float lr) {
   const int h = P->hidden, n = P->n;
-  cudaError_t e = enq_forward_chunk(P, P->X, B, true);
+  cudaError_t e = enq_hidden(P, P->X, B, true);
   if (e != cudaSuccess) return e;
-  if ((e = dlk::mlp_bce_grad(P->Z, B, n, P->sup, kPropMaxS, P->dZ, P->loss, P->st))) return e;
-  // layer 3
-  if ((e = dlk::mlp_transpose(P->dZ, B, n, P->dZt, P->st))) return e;
-  if ((e = dlk::mlp_transpose(P->H2, B, h, P->H2t, P->st))) return e;
-  if ((e = dlk::mlp_gemm(P->dZt, n, P->H2t, h, (int)B, dlk::MLP_EPI_F32, nullptr, nullptr, 0, P->g[4],
-                         nullptr, h, P->err, P->st)))
-    return e;
-  if ((e = dlk::mlp_colsum(P->dZ, B, n, P->g[5], P->st))) return e;
-  if ((e = dlk::mlp_transpose(P->wb[2], n, h, P->wt[1], P->st))) return e;
-  if ((e = dlk::mlp_gemm(P->dZ, B, P->wt[1], h, n, dlk::MLP_EPI_GELU_BWD, nullptr, P->A2, h, nullptr,
-                         P->dA2, h, P->err, P->st)))
-    return e;
-  // layer 2
-  if ((e = dlk::mlp_transpose(P->dA2, B, h, P->dA2t, P->st))) return e;
-  if ((e = dlk::mlp_transpose(P->H1, B, h, P->H1t, P->st))) return e;
-  if ((e = dlk::mlp_gemm(P->dA2t, h, P->H1t, h, (int)B, dlk::MLP_EPI_F32, nullptr, nullptr, 0, P->g[2],
-                         nullptr, h, P->err, P->st)))
-    return e;
-  if ((e = dlk::mlp_colsum(P->dA2, B, h, P->g[3], P->st))) return e;
-  if ((e = dlk::mlp_transpose(P->wb[1], h, h, P->wt[0], P->st))) return e;
-  if ((e = dlk::mlp_gemm(P->dA2, B, P->wt[0], h, h, dlk::MLP_EPI_GELU_BWD, nullptr, P->A1, h, nullptr,
-                         P->dA1, h, P->err, P->st)))
-    return e;
-  // layer 1
-  if ((e = dlk::mlp_transpose(P->dA1, B, h, P->dA1t, P->st))) return e;
-  if ((e = dlk::mlp_transpose(P->X, B, P->pk, P->Xt, P->st))) return e;
-  if ((e = dlk::mlp_gemm(P->dA1t, h, P->Xt, P->pk, (int)B, dlk::MLP_EPI_F32, nullptr, nullptr, 0,
-                         P->g[0], nullptr, P->pk, P->err, P->st)))
-    return e;
-  if ((e = dlk::mlp_colsum(P->dA1, B, h, P->g[1], P->st))) return e;
-  if (lr > 0.f) {
-    ++P->step;
-    for (int k = 0; k < 6; ++k)
-      if ((e = dlk::mlp_adam(P->w[k], P->g[k], P->am[k], P->av[k], P->wlen[k], lr, P->step,
-                             (k % 2 == 0) ? P->wb[k / 2] : nullptr, P->st)))
-        return e;
-  }
+  // output layer: its product, the loss, dZ and the bias gradient in one pass
+  dlk::MlpEpi ez{}, e2{}, e1{};
+  ez.bias = P->w[5];
+  ez.out_bf16 = (__nv_bfloat16*)P->dZ;
+  ez.ldc = n;
+  ez.colsum = P->g[5];
+  ez.sup = P->sup;
+  ez.loss = P->loss;
+  if ((e = dlk::mlp_forward(P->H2, B, P->wb[2], n, h, dlk::MLP_EPI_BCE, ez, P->err, P->st))) return e;
+  e2.aux = P->A2;
+  e2.out_bf16 = (__nv_bfloat16*)P->dA2;
+  e2.ldc = h;
+  e2.colsum = P->g[3];
+  if ((e = dlk::mlp_backward(P->dZ, B, P->wb[2], n, h, e2, P->H2, P->g[4], P->err, P->st))) return e;
+  e1.aux = P->A1;
+  e1.out_bf16 = (__nv_bfloat16*)P->dA1;
+  e1.ldc = h;
+  e1.colsum = P->g[1];
+  if ((e = dlk::mlp_backward(P->dA2, B, P->wb[1], h, h, e1, P->H1, P->g[2], P->err, P->st))) return e;
+  if ((e = dlk::mlp_backward_weight(P->dA1, P->X, B, h, P->pk, P->g[0], P->err, P->st))) return e;
+  if (lr > 0.f)
+    return dlk::mlp_adam(P->wall, P->gall, P->am, P->av, P->wpad, lr, ++P->step, P->wball, P->st);
   return cudaSuccess;
 }
 
@@ -1767,27 +1752,28 @@ extern "C" int dl_proposer_create(dl_proposer** out, int p, int n, int hidden, i
   P->st = (cudaStream_t)stream;
   const int64_t h = hidden, B = batch, BI = P->ichunk;
   const int64_t lens[6] = {h * P->pk, h, h * h, h, (int64_t)n * h, n};
-  bool ok = true;
-  for (int k = 0; k < 6 && ok; ++k) {
+  int64_t off[6];
+  for (int k = 0; k < 6; ++k) {  // every array on a 128-byte boundary in FP32 and BF16
     P->wlen[k] = lens[k];
-    ok = dalloc(&P->w[k], lens[k]) && dalloc(&P->g[k], lens[k]) && dalloc(&P->am[k], lens[k]) &&
-         dalloc(&P->av[k], lens[k]);
-    if (ok) ok = cudaMemset(P->w[k], 0, lens[k] * 4) == cudaSuccess &&
-                 cudaMemset(P->am[k], 0, lens[k] * 4) == cudaSuccess &&
-                 cudaMemset(P->av[k], 0, lens[k] * 4) == cudaSuccess;
+    off[k] = P->wpad;
+    P->wpad += (lens[k] + 63) / 64 * 64;
   }
+  const size_t wp = (size_t)P->wpad;
   const size_t b2 = 2;  // BF16 bytes
-  ok = ok && dalloc((uint8_t**)&P->wb[0], lens[0] * b2) && dalloc((uint8_t**)&P->wb[1], lens[2] * b2) &&
-       dalloc((uint8_t**)&P->wb[2], lens[4] * b2) && dalloc((uint8_t**)&P->wt[0], lens[2] * b2) &&
-       dalloc((uint8_t**)&P->wt[1], lens[4] * b2) && dalloc((uint8_t**)&P->X, B * P->pk * b2) &&
-       dalloc(&P->A1, B * h) && dalloc(&P->A2, B * h) && dalloc((uint8_t**)&P->H1, BI * h * b2) &&
-       dalloc((uint8_t**)&P->H2, BI * h * b2) && dalloc(&P->Z, B * n) &&
-       dalloc((uint8_t**)&P->Zb, BI * n * b2) && dalloc(&P->sup, B * kPropMaxS) &&
-       dalloc((uint8_t**)&P->dZ, B * n * b2) && dalloc((uint8_t**)&P->dZt, B * n * b2) &&
-       dalloc((uint8_t**)&P->H2t, B * h * b2) && dalloc((uint8_t**)&P->dA2, B * h * b2) &&
-       dalloc((uint8_t**)&P->dA2t, B * h * b2) && dalloc((uint8_t**)&P->H1t, B * h * b2) &&
-       dalloc((uint8_t**)&P->dA1, B * h * b2) && dalloc((uint8_t**)&P->dA1t, B * h * b2) &&
-       dalloc((uint8_t**)&P->Xt, B * P->pk * b2) && dalloc(&P->loss, 1) && dalloc(&P->err, 1) &&
+  bool ok = dalloc(&P->wall, wp) && dalloc(&P->gall, wp) && dalloc(&P->am, wp) && dalloc(&P->av, wp) &&
+            dalloc((uint8_t**)&P->wball, wp * b2) && cudaMemset(P->wall, 0, wp * 4) == cudaSuccess &&
+            cudaMemset(P->gall, 0, wp * 4) == cudaSuccess && cudaMemset(P->am, 0, wp * 4) == cudaSuccess &&
+            cudaMemset(P->av, 0, wp * 4) == cudaSuccess && cudaMemset(P->wball, 0, wp * b2) == cudaSuccess;
+  for (int k = 0; k < 6; ++k) {
+    P->w[k] = P->wall + off[k];
+    P->g[k] = P->gall + off[k];
+    if (k % 2 == 0) P->wb[k / 2] = (__nv_bfloat16*)P->wball + off[k];
+  }
+  ok = ok && dalloc((uint8_t**)&P->X, B * P->pk * b2) && dalloc(&P->A1, B * h) && dalloc(&P->A2, B * h) &&
+       dalloc((uint8_t**)&P->H1, BI * h * b2) && dalloc((uint8_t**)&P->H2, BI * h * b2) &&
+       dalloc(&P->Z, B * n) && dalloc((uint8_t**)&P->Zb, BI * n * b2) && dalloc(&P->sup, B * kPropMaxS) &&
+       dalloc((uint8_t**)&P->dZ, B * n * b2) && dalloc((uint8_t**)&P->dA2, B * h * b2) &&
+       dalloc((uint8_t**)&P->dA1, B * h * b2) && dalloc(&P->loss, 1) && dalloc(&P->err, 1) &&
        cudaMemset(P->err, 0, sizeof(int)) == cudaSuccess;
   if (!ok) {
     cudaGetLastError();
@@ -1815,11 +1801,9 @@ extern "C" int dl_proposer_set_weights(dl_proposer* P, const float* W1, const fl
   const float* src[6] = {nullptr, b1, W2, b2, W3, b3};
   for (int k = 1; k < 6; ++k)
     DL_CHECK(cudaMemcpyAsync(P->w[k], src[k], P->wlen[k] * 4, cudaMemcpyHostToDevice, P->st));
-  for (int k = 0; k < 3; ++k) DL_CHECK(dlk::mlp_to_bf16(P->w[2 * k], P->wlen[2 * k], P->wb[k], P->st));
-  for (int k = 0; k < 6; ++k) {
-    DL_CHECK(cudaMemsetAsync(P->am[k], 0, P->wlen[k] * 4, P->st));
-    DL_CHECK(cudaMemsetAsync(P->av[k], 0, P->wlen[k] * 4, P->st));
-  }
+  DL_CHECK(dlk::mlp_to_bf16(P->wall, P->wpad, P->wball, P->st));
+  DL_CHECK(cudaMemsetAsync(P->am, 0, P->wpad * 4, P->st));
+  DL_CHECK(cudaMemsetAsync(P->av, 0, P->wpad * 4, P->st));
   P->step = 0;
   DL_CHECK(cudaStreamSynchronize(P->st));
   return DL_OK;
@@ -1849,11 +1833,8 @@ extern "C" int dl_proposer_train(dl_proposer* P, const float* Y, int64_t m, cons
   DL_CHECK(cudaMemsetAsync(P->loss, 0, sizeof(double), P->st));
   int64_t steps = 0;
   for (int64_t r0 = 0; r0 + batch <= m; r0 += batch, ++steps) {
-    const int64_t tot = batch * P->pk;
-    gather_rows_kernel<<<(unsigned)((tot + 255) / 256), 256, 0, P->st>>>(
-        perm ? Y : Y + r0 * P->p, P->p, P->pk, perm ? perm + r0 : nullptr, batch, perm ? sup : sup + r0 * s,
-        s, (__nv_bfloat16*)P->X, P->sup);
-    DL_CHECK(cudaGetLastError());
+    DL_CHECK(dlk::mlp_gather(perm ? Y : Y + r0 * P->p, P->p, P->pk, perm ? perm + r0 : nullptr, batch,
+                             perm ? sup : sup + r0 * s, s, P->X, P->sup, P->gall, P->wpad, P->st));
     DL_CHECK(enq_train_step(P, batch, lr));
   }
   if (steps == 0) return DL_EINVAL;
@@ -1875,19 +1856,13 @@ extern "C" int dl_proposer_forward(dl_proposer* P, const float* Y, int64_t m, fl
   DevGuard g(P->dev);
   for (int64_t r0 = 0; r0 < m; r0 += P->bmax) {
     const int64_t B = m - r0 < P->bmax ? m - r0 : P->bmax;
-    const int64_t tot = B * P->pk;
-    gather_rows_kernel<<<(unsigned)((tot + 255) / 256), 256, 0, P->st>>>(
-        Y + r0 * P->p, P->p, P->pk, nullptr, B, nullptr, 0, (__nv_bfloat16*)P->X, nullptr);
-    DL_CHECK(cudaGetLastError());
-    if (logits) {
-      DL_CHECK(enq_forward_chunk(P, P->X, B, true));
+    DL_CHECK(dlk::mlp_gather(Y + r0 * P->p, P->p, P->pk, nullptr, B, nullptr, 0, P->X, nullptr, nullptr, 0,
+                             P->st));
+    DL_CHECK(enq_logits(P, P->X, B, logits ? P->Z : nullptr, cand ? P->Zb : nullptr));
+    if (logits)
       DL_CHECK(cudaMemcpyAsync(logits + r0 * P->n, P->Z, sizeof(float) * B * P->n,
                                cudaMemcpyDeviceToDevice, P->st));
-    }
-    if (cand) {
-      DL_CHECK(enq_forward_chunk(P, P->X, B, false));
-      DL_CHECK(dlk::mlp_topk(P->Zb, B, P->n, K, cand + r0 * K, P->st));
-    }
+    if (cand) DL_CHECK(dlk::mlp_topk(P->Zb, B, P->n, K, cand + r0 * K, P->st));
   }
   DL_CHECK(cudaStreamSynchronize(P->st));
   return DL_OK;

@@ -2,6 +2,7 @@
 // Nothing here is part of the public C ABI (include/dl_gb300.h).
 #pragma once
 
+#include <cuda_bf16.h>
 #include <cuda_runtime.h>
 #include <stdint.h>
 
@@ -146,17 +147,33 @@ cudaError_t omp_listed(const int* list, const int* count, const float* A0, int64
                        cudaStream_t st);
 
 // ---- learned proposer (k_mlp.cu) ----------------------------------------------
-enum : int { MLP_EPI_BF16 = 0, MLP_EPI_F32 = 1, MLP_EPI_GELU_FWD = 2, MLP_EPI_GELU_BWD = 3 };
+enum : int { MLP_EPI_GELU_FWD, MLP_EPI_LOGITS, MLP_EPI_BCE, MLP_EPI_GELU_BWD, MLP_EPI_RED };
+struct MlpEpi {
+  const float* bias;        // [N] or null
+  const float* aux;         // GELU_BWD: pre-activation (FP32, ld = ldc)
+  float* out_f32;           // LOGITS: logits; GELU_FWD: pre-activation; or null; RED: summed into
+  __nv_bfloat16* out_bf16;  // BF16 output (LOGITS: or null)
+  int64_t ldc;              // row length of the outputs and aux
+  float* colsum;            // GELU_BWD, BCE: column sums of the BF16 output are added here
+  const int32_t* sup;       // BCE: 16 support slots per row (-1: none)
+  double* loss;             // BCE: the mean loss is added here
+};
 bool mlp_gemm_supported();
-// C[M x N] = A[M x K] B[N x K]^T, BF16 row-major operands (K % 64 == 0), epilogue op.
-cudaError_t mlp_gemm(const void* A, int64_t M, const void* B, int N, int K, int op, const float* bias,
-                     const float* aux, int64_t ldaux, float* out_f32, void* out_bf16, int64_t ldc,
-                     int* err, cudaStream_t st);
-cudaError_t mlp_transpose(const void* in, int64_t R, int64_t C, void* out, cudaStream_t st);
+// out = op(A W^T): A M x K, W N x K, BF16 (K % 64 == 0, N % 64 == 0).
+cudaError_t mlp_forward(const void* A, int64_t M, const void* W, int N, int K, int op,
+                        const MlpEpi& epi, int* err, cudaStream_t st);
+// One launch: out = (dY W) * gelu'(aux) (dY B x Nout, W Nout x Nin), and
+// dW (zeroed by the caller) += dY^T X (X B x Nin).
+cudaError_t mlp_backward(const void* dY, int64_t B, const void* W, int Nout, int Nin, const MlpEpi& epi,
+                         const void* X, float* dW, int* err, cudaStream_t st);
+// Rows of Y (selected by idx when given) as BF16 rows pk wide, their support slots
+// (16 per row) when sup_in is given, and zero_len floats (a multiple of 4) cleared.
+cudaError_t mlp_gather(const float* Y, int p, int pk, const int64_t* idx, int64_t B, const int32_t* sup_in,
+                       int s, void* X, int32_t* sup_out, float* zero, int64_t zero_len, cudaStream_t st);
+// dW (Nout x Nin, zeroed by the caller) += dY^T X: dY B x Nout, X B x Nin.
+cudaError_t mlp_backward_weight(const void* dY, const void* X, int64_t B, int Nout, int Nin, float* dW,
+                                int* err, cudaStream_t st);
 cudaError_t mlp_to_bf16(const float* in, int64_t count, void* out, cudaStream_t st);
-cudaError_t mlp_bce_grad(const float* z, int64_t B, int n, const int32_t* sup, int s, void* dz,
-                         double* loss, cudaStream_t st);
-cudaError_t mlp_colsum(const void* in, int64_t R, int C, float* out, cudaStream_t st);
 cudaError_t mlp_adam(float* w, const float* g, float* m, float* v, int64_t count, float lr, int t,
                      void* wbf, cudaStream_t st);
 cudaError_t mlp_topk(const void* z, int64_t m, int n, int K, int32_t* cand, cudaStream_t st);

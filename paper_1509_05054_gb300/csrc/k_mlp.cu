@@ -1,10 +1,22 @@
-// The learned support proposer: a BF16 MLP p -> 512 -> 512 -> n (GELU, sigmoid
+// The learned support proposer: a BF16 MLP p -> hidden -> hidden -> n (GELU, sigmoid
 // outputs) trained with binary cross-entropy on multi-hot OMP supports, and its
 // inference (top-2s candidates per signal).  All products run on one tcgen05
-// GEMM kernel, C = A B^T with BF16 operands stored row-major with K contiguous,
-// FP32 accumulation in TMEM and fused epilogues (bias, GELU, GELU derivative,
-// BF16 or FP32 output).  Backward products that contract over the batch use
-// explicitly transposed BF16 copies, so every operand stays K-major.
+// GEMM kernel with FP32 accumulation in TMEM and fused epilogues (bias, GELU,
+// GELU derivative, the cross-entropy's gradient and loss, bias gradients).
+// Operands are BF16, row-major; either may be contracted along its rows
+// (K-major tiles) or along its columns (MN-major tiles), so the backward
+// products read the forward pass's arrays as they are.
+//
+// What bounds a training step of 4096 rows at hidden = n = 512 (13 GFLOP, 7 us of
+// tensor time) is everything around the MMAs.  Measured before (us per step):
+// products 258 (64 CTAs of 128 threads, a row per thread in the epilogue, scalar
+// atomics for the split sums), the loss and its gradient as a kernel with
+// FP64 arithmetic per element 68, explicit transposes 37, column sums 29, six
+// memsets 8; with the gaps 460.  Now 77: seven launches that overlap each other's
+// start, 128 x 128 tiles with sixteen warps and coalesced rows in the epilogue, the
+// loss, its gradient and the bias gradients in the epilogues, vector reductions for
+// the split sums, and a layer's two backward products in one launch.  What is left is
+// mostly each launch's chain of load, MMA and epilogue latencies (about 10 us).
 #include "dl_internal.cuh"
 #include "tc_ptx.cuh"
 
@@ -19,15 +31,20 @@ namespace {
 
 using namespace tc;
 
-constexpr int GM_THREADS = 128;
-constexpr int GM_TILE_M = 128;
-constexpr int GM_BLOCK_N = 256;
-constexpr int GM_BK = 64;  // BF16 elements per 128-byte chunk
-constexpr int GM_STAGES = 4;
-constexpr size_t GM_A_BYTES = (size_t)GM_TILE_M * 128;   // 16 KB
-constexpr size_t GM_B_BYTES = (size_t)GM_BLOCK_N * 128;  // 32 KB
-constexpr uint32_t kIdescBf16 = (1u << 4) | (1u << 7) | (1u << 10) |
-                                ((uint32_t)(GM_BLOCK_N >> 3) << 17) | ((uint32_t)(GM_TILE_M >> 4) << 24);
+constexpr int GM_THREADS = 512;  // sixteen warps: four per TMEM lane quadrant in the epilogue
+constexpr int GM_TILE = 128;     // rows and columns of a CTA's output tile
+constexpr int GM_BK = 64;        // contraction elements per stage (128 bytes of BF16)
+constexpr int GM_WC = GM_TILE / (GM_THREADS / 128);  // columns a warp takes in the epilogue (of 32 rows)
+constexpr int GM_WU = GM_WC / 4;                     // as 16-byte units
+// Three stages of 32 KB: two CTAs per SM, so that one's epilogue overlaps the
+// other's loads and MMAs.
+constexpr int GM_STAGES = 3;
+constexpr uint32_t GM_OP_BYTES = GM_TILE * GM_BK * 2;  // one operand of a stage, 16 KB
+constexpr size_t GM_SMEM = 1024 + (size_t)GM_STAGES * 2 * GM_OP_BYTES + 256;
+static_assert((size_t)GM_STAGES * 2 * GM_OP_BYTES >= GM_TILE * GM_TILE * sizeof(float), "epilogue staging");
+// kind::f16: D F32, A and B BF16, M = N = 128; bits 15 and 16: A, B MN-major
+constexpr uint32_t kIdesc = (1u << 4) | (1u << 7) | (1u << 10) | ((uint32_t)(GM_TILE >> 3) << 17) |
+                            ((uint32_t)(GM_TILE >> 4) << 24);
 
 __device__ __forceinline__ float gelu_f(float a) { return 0.5f * a * (1.f + erff(a * 0.70710678118654752f)); }
 __device__ __forceinline__ float gelu_grad_f(float a) {
@@ -35,35 +52,88 @@ __device__ __forceinline__ float gelu_grad_f(float a) {
          a * 0.39894228040143268f * expf(-0.5f * a * a);
 }
 
-struct Epi {
-  int op;                  // MLP_EPI_*
-  const float* bias;       // [N] or null
-  const float* aux;        // GELU_BWD: pre-activation [M x ldaux] (FP32)
-  int64_t ldaux;
-  float* out_f32;          // F32 output (and pre-activation for GELU_FWD), ld = ldc
-  __nv_bfloat16* out_bf16; // BF16 output, ld = ldc
-  int64_t ldc;
+// Descriptor of an operand tile: K-major (128 rows of 128 bytes), or MN-major
+// (two blocks of 64 columns, 8 KB apart, each 64 contraction rows of 128 bytes),
+// both with the 128-byte swizzle and 8-row groups of 1024 bytes.
+template <bool MN>
+__device__ __forceinline__ uint64_t tile_desc(const void* base) {
+  uint64_t d = sw128_desc(base);
+  if (MN) d += (uint64_t)((8192 >> 4) - 1) << 16;  // leading byte offset
+  return d;
+}
+// 16 contraction elements further (descriptor units of 16 bytes).
+template <bool MN>
+constexpr uint64_t kstep() { return MN ? (16 * 128) >> 4 : 32 >> 4; }
+
+template <bool MN>
+__device__ __forceinline__ void load_tile(uint8_t* dst, const CUtensorMap* map, uint64_t* bar, int k0,
+                                          int mn0) {
+  if (MN) {
+    tma_load_2d(dst, map, bar, mn0, k0);
+    tma_load_2d(dst + 8192, map, bar, mn0 + 64, k0);
+  } else {
+    tma_load_2d(dst, map, bar, k0, mn0);
+  }
+}
+
+// Sum of FP32 values kept as an unevaluated pair (Knuth's two-sum: the rounding
+// error of every addition goes to lo), so that FP64 is needed once per thread.
+struct Sum2 {
+  float hi = 0.f, lo = 0.f;
+  __device__ __forceinline__ void add(float x) {
+    const float s = __fadd_rn(hi, x), b = __fsub_rn(s, hi);
+    lo += __fadd_rn(__fsub_rn(hi, __fsub_rn(s, b)), __fsub_rn(x, b));
+    hi = s;
+  }
 };
 
-// C[M x N] = A[M x K] B[N x K]^T ; one CTA per (128-row tile, 256-column block).
-__global__ void __launch_bounds__(GM_THREADS, 1)
-    gemm_bf16_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ CUtensorMap tmB,
-                     int64_t M, int N, int K, Epi epi, int* __restrict__ err) {
-  // blockIdx.z selects a slice of the K chunks (split-K; F32 output accumulated atomically)
+__device__ __forceinline__ uint2 pack_bf16x4(float4 v) {
+  const __nv_bfloat162 a = __floats2bfloat162_rn(v.x, v.y), b = __floats2bfloat162_rn(v.z, v.w);
+  return make_uint2(*(const uint32_t*)&a, *(const uint32_t*)&b);
+}
+
+// C[M x N] = A B, contraction length K: A is M x K (AMN: stored K x M), B is N x K
+// (BMN: stored K x N), row-major BF16; M or N or K need not fill the tiles (TMA
+// fills with zeros), N % 64 == 0, K % 64 == 0.  One CTA per 128 x 128 tile and
+// slice bz of the contraction.  Warp 0 issues the TMA loads, warp 1 the
+// MMAs; then all sixteen warps take 32 rows x 32 columns each through shared memory
+// (16-byte units XORed with the row: no bank conflicts either way) so that every
+// global access is whole 128-byte lines (FP32) and a lane keeps the same four
+// columns throughout.
+struct Job {
+  CUtensorMap A, B;
+  int64_t M;
+  int N, K;
+  int gx, gy, gz;  // row tiles, column tiles, slices of the contraction
+  MlpEpi epi;
+};
+
+template <bool AMN, bool BMN, int OP>
+__device__ __forceinline__ void gemm_tile(const Job& job, int bx, int by, int bz, int* __restrict__ err) {
+  const CUtensorMap& tmA = job.A;
+  const CUtensorMap& tmB = job.B;
+  const int64_t M = job.M;
+  const int N = job.N, K = job.K;
+  const MlpEpi& epi = job.epi;
   extern __shared__ uint8_t smem_raw[];
   uint8_t* base = (uint8_t*)(((uintptr_t)smem_raw + 1023) & ~(uintptr_t)1023);
   uint8_t* As = base;
-  uint8_t* Bs = base + GM_STAGES * GM_A_BYTES;
-  uint64_t* full = (uint64_t*)(Bs + GM_STAGES * GM_B_BYTES);
+  uint8_t* Bs = base + GM_STAGES * GM_OP_BYTES;
+  uint64_t* full = (uint64_t*)(Bs + GM_STAGES * GM_OP_BYTES);
   uint64_t* empty = full + GM_STAGES;
   uint64_t* done = empty + GM_STAGES;
   uint32_t* tmem_slot = (uint32_t*)(done + 1);
   __shared__ int s_fail;
+  __shared__ double s_loss[GM_THREADS / 32];
 
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-  const int64_t m0 = (int64_t)blockIdx.x * GM_TILE_M;
-  const int n0 = blockIdx.y * GM_BLOCK_N;
+  const int64_t m0 = (int64_t)bx * GM_TILE;
+  const int n0 = by * GM_TILE;
   const int nk = K / GM_BK;
+  const int per = (nk + job.gz - 1) / job.gz;
+  const int kbeg = bz * per;
+  const int cnt = (kbeg + per < nk ? kbeg + per : nk) - kbeg;
+  if (cnt <= 0) return;  // no share of the contraction (uniform in the CTA)
 
   if (threadIdx.x == 0) {
     s_fail = 0;
@@ -77,7 +147,7 @@ __global__ void __launch_bounds__(GM_THREADS, 1)
   if (warp == 0) {
     asm volatile("tcgen05.alloc.cta_group::1.sync.aligned.shared::cta.b32 [%0], %1;" ::"r"(
                      smem_u32(tmem_slot)),
-                 "r"(256u)
+                 "r"((uint32_t)GM_TILE)
                  : "memory");
     asm volatile("tcgen05.relinquish_alloc_permit.cta_group::1.sync.aligned;" ::: "memory");
   }
@@ -85,41 +155,38 @@ __global__ void __launch_bounds__(GM_THREADS, 1)
   __syncthreads();
   tc_fence_after();
   const uint32_t tmem = *tmem_slot;
+  // The setup above overlaps the end of the previous kernel (launch_gemm): the
+  // next one may start its own, and nothing before this wait reads or writes
+  // global memory.
+  asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
+  asm volatile("griddepcontrol.wait;" ::: "memory");
 
-  const int kz = (int)gridDim.z;
-  const int per = (nk + kz - 1) / kz;
-  const int kbeg = (int)blockIdx.z * per;
-  const int kend = kbeg + per < nk ? kbeg + per : nk;
-  const int cnt = kend > kbeg ? kend - kbeg : 0;
   if (threadIdx.x == 0) {
-    bool ok = true;
-    for (int q = 0; q < GM_STAGES && q < cnt; ++q) {
-      mbar_expect_tx(&full[q], (uint32_t)(GM_A_BYTES + GM_B_BYTES));
-      tma_load_2d(As + q * GM_A_BYTES, &tmA, &full[q], (kbeg + q) * GM_BK, (int)m0);
-      tma_load_2d(Bs + q * GM_B_BYTES, &tmB, &full[q], (kbeg + q) * GM_BK, n0);
+    for (int j = 0; j < cnt; ++j) {
+      const int st = j % GM_STAGES;
+      if (j >= GM_STAGES && !mbar_wait(&empty[st], (uint32_t)((j / GM_STAGES - 1) & 1))) {
+        s_fail = 1;
+        break;
+      }
+      mbar_expect_tx(&full[st], 2 * GM_OP_BYTES);
+      load_tile<AMN>(As + st * GM_OP_BYTES, &tmA, &full[st], (kbeg + j) * GM_BK, (int)m0);
+      load_tile<BMN>(Bs + st * GM_OP_BYTES, &tmB, &full[st], (kbeg + j) * GM_BK, n0);
     }
-    for (int j = 0; j < cnt && ok; ++j) {
+  } else if (threadIdx.x == 32) {
+    bool ok = true;
+    for (int j = 0; j < cnt; ++j) {
       const int st = j % GM_STAGES;
       if (!(ok = mbar_wait(&full[st], (uint32_t)((j / GM_STAGES) & 1)))) break;
       tc_fence_after();
-      const uint64_t ad = sw128_desc(As + st * GM_A_BYTES);
-      const uint64_t bd = sw128_desc(Bs + st * GM_B_BYTES);
+      const uint64_t ad = tile_desc<AMN>(As + st * GM_OP_BYTES);
+      const uint64_t bd = tile_desc<BMN>(Bs + st * GM_OP_BYTES);
 #pragma unroll
-      for (int k = 0; k < 4; ++k)
-        mma_f16(tmem, ad + (uint64_t)(2 * k), bd + (uint64_t)(2 * k), kIdescBf16,
-                (j > 0 || k > 0) ? 1u : 0u);
+      for (int k = 0; k < GM_BK / 16; ++k)
+        mma_f16(tmem, ad + k * kstep<AMN>(), bd + k * kstep<BMN>(),
+                kIdesc | (AMN ? 1u << 15 : 0u) | (BMN ? 1u << 16 : 0u), (j > 0 || k > 0) ? 1u : 0u);
       mma_commit(&empty[st]);
-      // refill the stage of the previous chunk (its MMAs were issued one step ago)
-      const int jp = j - 1, jn = jp + GM_STAGES;
-      if (jp >= 0 && jn < cnt) {
-        const int ps = jp % GM_STAGES;
-        if (!(ok = mbar_wait(&empty[ps], (uint32_t)((jp / GM_STAGES) & 1)))) break;
-        mbar_expect_tx(&full[ps], (uint32_t)(GM_A_BYTES + GM_B_BYTES));
-        tma_load_2d(As + ps * GM_A_BYTES, &tmA, &full[ps], (kbeg + jn) * GM_BK, (int)m0);
-        tma_load_2d(Bs + ps * GM_B_BYTES, &tmB, &full[ps], (kbeg + jn) * GM_BK, n0);
-      }
     }
-    if (ok && cnt > 0) {
+    if (ok) {
       mma_commit(done);
       ok = mbar_wait(done, 0);
     }
@@ -127,87 +194,146 @@ __global__ void __launch_bounds__(GM_THREADS, 1)
   }
   __syncthreads();
   tc_fence_after();
-  if (!s_fail && cnt > 0) {
-    const int64_t row = m0 + warp * 32 + lane;
-    const uint32_t lane_base = (uint32_t)(warp * 32) << 16;
-    const int ncols = N - n0 < GM_BLOCK_N ? N - n0 : GM_BLOCK_N;
-    const bool split = kz > 1;
-    for (int c0 = 0; c0 < ncols; c0 += 16) {
+  double loss = 0.0;
+  const int col0 = n0 + GM_WC * (warp >> 2);
+  if (!s_fail && col0 < N) {
+    const int quad = warp & 3;
+    float4* stage = (float4*)base + warp * (32 * GM_WU);
+#pragma unroll
+    for (int c = 0; c < GM_WC / 16; ++c) {
       uint32_t r[16];
-      tmem_ld16(tmem + lane_base + (uint32_t)c0, r);
-      if (row >= M) continue;
-      const int col0 = n0 + c0;
-      const bool full16 = col0 + 16 <= N && (epi.ldc % 8) == 0;
-      float a[16], o[16];
+      tmem_ld16(tmem + ((uint32_t)(quad * 32) << 16) + (uint32_t)(GM_WC * (warp >> 2) + 16 * c), r);
 #pragma unroll
-      for (int q = 0; q < 16; ++q) {
-        a[q] = __uint_as_float(r[q]);
-        if (epi.bias && !split && col0 + q < N) a[q] += epi.bias[col0 + q];
-      }
-      if (epi.op == MLP_EPI_F32) {
-        float* dst = epi.out_f32 + row * epi.ldc + col0;
-        if (split) {
+      for (int q = 0; q < 4; ++q)
+        stage[lane * GM_WU + ((4 * c + q) ^ (lane & (GM_WU - 1)))] =
+            make_float4(__uint_as_float(r[4 * q]), __uint_as_float(r[4 * q + 1]),
+                        __uint_as_float(r[4 * q + 2]), __uint_as_float(r[4 * q + 3]));
+    }
+    const int64_t row0 = m0 + quad * 32;
+    const int u = lane & (GM_WU - 1), rl = lane / GM_WU, col = col0 + 4 * u;
+    uint32_t target = 0;  // BCE: lane = row, its support inside these 32 columns
+    if (OP == MLP_EPI_BCE && row0 + lane < M) {
+      static_assert(GM_WC == 32, "target bits");
+      const int4* sp = (const int4*)(epi.sup + (row0 + lane) * 16);
 #pragma unroll
-          for (int q = 0; q < 16; ++q)
-            if (col0 + q < N) atomicAdd(dst + q, a[q]);
-        } else if (full16) {
-#pragma unroll
-          for (int q = 0; q < 4; ++q)
-            ((float4*)dst)[q] = make_float4(a[4 * q], a[4 * q + 1], a[4 * q + 2], a[4 * q + 3]);
-        } else {
-#pragma unroll
-          for (int q = 0; q < 16; ++q)
-            if (col0 + q < N) dst[q] = a[q];
-        }
-        continue;
-      }
-      if (epi.op == MLP_EPI_GELU_FWD) {
-        if (epi.out_f32) {
-          float* pre = epi.out_f32 + row * epi.ldc + col0;
-          if (full16) {
-#pragma unroll
-            for (int q = 0; q < 4; ++q)
-              ((float4*)pre)[q] = make_float4(a[4 * q], a[4 * q + 1], a[4 * q + 2], a[4 * q + 3]);
-          } else {
-#pragma unroll
-            for (int q = 0; q < 16; ++q)
-              if (col0 + q < N) pre[q] = a[q];
-          }
-        }
-#pragma unroll
-        for (int q = 0; q < 16; ++q) o[q] = gelu_f(a[q]);
-      } else if (epi.op == MLP_EPI_GELU_BWD) {
-        const float* aux = epi.aux + row * epi.ldaux + col0;
-#pragma unroll
-        for (int q = 0; q < 16; ++q) o[q] = (col0 + q < N) ? a[q] * gelu_grad_f(aux[q]) : 0.f;
-      } else {
-#pragma unroll
-        for (int q = 0; q < 16; ++q) o[q] = a[q];
-      }
-      __nv_bfloat16* dst = epi.out_bf16 + row * epi.ldc + col0;
-      if (full16) {
-        uint32_t w[8];
-#pragma unroll
-        for (int q = 0; q < 8; ++q) {
-          const __nv_bfloat162 h2 = __floats2bfloat162_rn(o[2 * q], o[2 * q + 1]);
-          w[q] = *(const uint32_t*)&h2;
-        }
-        ((uint4*)dst)[0] = make_uint4(w[0], w[1], w[2], w[3]);
-        ((uint4*)dst)[1] = make_uint4(w[4], w[5], w[6], w[7]);
-      } else {
-#pragma unroll
-        for (int q = 0; q < 16; ++q)
-          if (col0 + q < N) dst[q] = __float2bfloat16_rn(o[q]);
+      for (int q = 0; q < 4; ++q) {
+        const int4 v = __ldg(sp + q);
+        if ((unsigned)(v.x - col0) < 32u) target |= 1u << (v.x - col0);
+        if ((unsigned)(v.y - col0) < 32u) target |= 1u << (v.y - col0);
+        if ((unsigned)(v.z - col0) < 32u) target |= 1u << (v.z - col0);
+        if ((unsigned)(v.w - col0) < 32u) target |= 1u << (v.w - col0);
       }
     }
-  } else if (threadIdx.x == 0) {
-    atomicOr(err, ERR_TIMEOUT);
+    const float4 bias = epi.bias ? __ldg((const float4*)(epi.bias + col)) : make_float4(0.f, 0.f, 0.f, 0.f);
+    const float fm = (float)M, im = 1.f / fm;
+    const bool pow2 = (M & (M - 1)) == 0;  // then the product with 1/M is the quotient, exactly
+    float4 cs = make_float4(0.f, 0.f, 0.f, 0.f);  // column sums of the BF16 output
+    Sum2 ls;
+    __syncwarp();
+#pragma unroll 2
+    for (int it = 0; it < GM_WU; ++it) {
+      const int rr = (32 / GM_WU) * it + rl;
+      const int64_t row = row0 + rr;
+      const uint32_t tg = OP == MLP_EPI_BCE ? __shfl_sync(0xffffffffu, target, rr) >> (4 * u) : 0;
+      if (row >= M) continue;
+      float4 a = stage[rr * GM_WU + (u ^ (rr & (GM_WU - 1)))];
+      const int64_t o = row * epi.ldc + col;
+      if (OP == MLP_EPI_RED) {
+        asm volatile("red.global.add.v4.f32 [%0], {%1, %2, %3, %4};" ::"l"(epi.out_f32 + o), "f"(a.x),
+                     "f"(a.y), "f"(a.z), "f"(a.w)
+                     : "memory");
+        continue;
+      }
+      a.x += bias.x;
+      a.y += bias.y;
+      a.z += bias.z;
+      a.w += bias.w;
+      if (OP == MLP_EPI_LOGITS || OP == MLP_EPI_GELU_FWD)
+        if (epi.out_f32) *(float4*)(epi.out_f32 + o) = a;
+      if (OP == MLP_EPI_GELU_FWD) {
+        a = make_float4(gelu_f(a.x), gelu_f(a.y), gelu_f(a.z), gelu_f(a.w));
+      } else if (OP == MLP_EPI_GELU_BWD) {
+        const float4 x = __ldg((const float4*)(epi.aux + o));
+        a = make_float4(a.x * gelu_grad_f(x.x), a.y * gelu_grad_f(x.y), a.z * gelu_grad_f(x.z),
+                        a.w * gelu_grad_f(x.w));
+      } else if (OP == MLP_EPI_BCE) {
+        // dz = (sigmoid(z) - t) / B, and the loss sum(softplus(z) - t z) / B
+        float* v = &a.x;
+#pragma unroll
+        for (int q = 0; q < 4; ++q) {
+          const float z = v[q], t = (tg >> q & 1) ? 1.f : 0.f;
+          const float sg = 1.f / (1.f + expf(-z));
+          const float sp = fmaxf(z, 0.f) + log1pf(expf(-fabsf(z)));
+          ls.add(sp - t * z);
+          v[q] = pow2 ? (sg - t) * im : (sg - t) / fm;
+        }
+      }
+      if (OP != MLP_EPI_LOGITS || epi.out_bf16) {
+        const uint2 h = pack_bf16x4(a);
+        *(uint2*)(epi.out_bf16 + o) = h;
+        if (OP == MLP_EPI_GELU_BWD || OP == MLP_EPI_BCE) {
+          cs.x += __uint_as_float(h.x << 16);
+          cs.y += __uint_as_float(h.x & 0xffff0000u);
+          cs.z += __uint_as_float(h.y << 16);
+          cs.w += __uint_as_float(h.y & 0xffff0000u);
+        }
+      }
+    }
+    if (OP == MLP_EPI_GELU_BWD || OP == MLP_EPI_BCE) {
+#pragma unroll
+      for (int o = GM_WU; o < 32; o <<= 1) {
+        cs.x += __shfl_xor_sync(0xffffffffu, cs.x, o);
+        cs.y += __shfl_xor_sync(0xffffffffu, cs.y, o);
+        cs.z += __shfl_xor_sync(0xffffffffu, cs.z, o);
+        cs.w += __shfl_xor_sync(0xffffffffu, cs.w, o);
+      }
+      if (lane < GM_WU)
+        asm volatile("red.global.add.v4.f32 [%0], {%1, %2, %3, %4};" ::"l"(epi.colsum + col), "f"(cs.x),
+                     "f"(cs.y), "f"(cs.z), "f"(cs.w)
+                     : "memory");
+    }
+    if (OP == MLP_EPI_BCE) loss = (double)ls.hi + (double)ls.lo;
   }
+  if (OP == MLP_EPI_BCE) {
+#pragma unroll
+    for (int o = 16; o > 0; o >>= 1) loss += __shfl_xor_sync(0xffffffffu, loss, o);
+    if (lane == 0) s_loss[warp] = loss;
+  }
+  if (s_fail && threadIdx.x == 0) atomicOr(err, ERR_TIMEOUT);
   tc_fence_before();
   __syncthreads();
+  if (OP == MLP_EPI_BCE && threadIdx.x == 0) {
+    for (int w = 1; w < GM_THREADS / 32; ++w) loss += s_loss[w];
+    atomicAdd(epi.loss, loss / (double)M);
+  }
   if (warp == 0)
-    asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;" ::"r"(tmem), "r"(256u)
+    asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;" ::"r"(tmem),
+                 "r"((uint32_t)GM_TILE)
                  : "memory");
+}
+
+template <bool AMN, bool BMN, int OP>
+__global__ void __launch_bounds__(GM_THREADS, 2)
+    gemm_bf16_kernel(const __grid_constant__ Job job, int* __restrict__ err) {
+  const int t = (int)blockIdx.x % (job.gx * job.gy);
+  gemm_tile<AMN, BMN, OP>(job, t % job.gx, t / job.gx, (int)blockIdx.x / (job.gx * job.gy), err);
+}
+
+// A layer's two backward products, which read the same dY, in one launch: the
+// input gradient dY W (with the GELU derivative), then the weight gradient
+// dY^T X.  Either alone leaves a good part of the two CTAs per SM idle (128 and
+// 144 CTAs of 304 at batch 4096 and width 512).
+__global__ void __launch_bounds__(GM_THREADS, 2)
+    gemm_backward_kernel(const __grid_constant__ Job data, const __grid_constant__ Job weight,
+                         int* __restrict__ err) {
+  const int nd = data.gx * data.gy, b = (int)blockIdx.x;
+  if (b < nd) {
+    gemm_tile<false, true, MLP_EPI_GELU_BWD>(data, b % data.gx, b / data.gx, 0, err);
+  } else {
+    const int t = (b - nd) % (weight.gx * weight.gy);
+    gemm_tile<true, true, MLP_EPI_RED>(weight, t % weight.gx, t / weight.gx,
+                                       (b - nd) / (weight.gx * weight.gy), err);
+  }
 }
 
 PFN_cuTensorMapEncodeTiled_v12000 encode_fn() {
@@ -223,11 +349,12 @@ PFN_cuTensorMapEncodeTiled_v12000 encode_fn() {
   return fn;
 }
 
-bool map_bf16(CUtensorMap* map, const void* ptr, int64_t rows, int K, int box_rows) {
+// rows x cols BF16, row-major; boxes of 64 columns (128 bytes) x box_rows.
+bool map_bf16(CUtensorMap* map, const void* ptr, int64_t rows, int64_t cols, int box_rows) {
   auto fn = encode_fn();
   if (!fn) return false;
-  cuuint64_t dims[2] = {(cuuint64_t)K, (cuuint64_t)rows};
-  cuuint64_t strides[1] = {(cuuint64_t)K * 2};
+  cuuint64_t dims[2] = {(cuuint64_t)cols, (cuuint64_t)rows};
+  cuuint64_t strides[1] = {(cuuint64_t)cols * 2};
   cuuint32_t box[2] = {(cuuint32_t)GM_BK, (cuuint32_t)box_rows};
   cuuint32_t estr[2] = {1, 1};
   return fn(map, CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, 2, (void*)ptr, dims, strides, box, estr,
@@ -235,70 +362,88 @@ bool map_bf16(CUtensorMap* map, const void* ptr, int64_t rows, int K, int box_ro
             CU_TENSOR_MAP_L2_PROMOTION_L2_256B, CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE) == CUDA_SUCCESS;
 }
 
-// [R x C] BF16 -> [C x R] BF16 through 32 x 32 shared-memory tiles.
-__global__ void transpose_bf16_kernel(const __nv_bfloat16* __restrict__ in, int64_t R, int64_t C,
-                                      __nv_bfloat16* __restrict__ out) {
-  __shared__ __nv_bfloat16 tile[32][33];
-  const int64_t c0 = (int64_t)blockIdx.x * 32, r0 = (int64_t)blockIdx.y * 32;
-  for (int k = threadIdx.y; k < 32; k += blockDim.y) {
-    const int64_t r = r0 + k, c = c0 + threadIdx.x;
-    if (r < R && c < C) tile[k][threadIdx.x] = in[r * C + c];
+bool make_job(Job& j, bool amn, const void* A, int64_t M, bool bmn, const void* B, int N, int64_t K,
+              int slices, const MlpEpi& epi) {
+  if (K <= 0 || K % GM_BK != 0 || N % 64 != 0) return false;
+  j.M = M;
+  j.N = N;
+  j.K = (int)K;
+  j.gx = (int)((M + GM_TILE - 1) / GM_TILE);
+  j.gy = (N + GM_TILE - 1) / GM_TILE;
+  j.gz = slices;
+  j.epi = epi;
+  return (amn ? map_bf16(&j.A, A, K, M, GM_BK) : map_bf16(&j.A, A, M, K, GM_TILE)) &&
+         (bmn ? map_bf16(&j.B, B, K, N, GM_BK) : map_bf16(&j.B, B, N, K, GM_TILE));
+}
+
+// Programmatic dependent launch: the kernel's barriers, TMEM and launch latency
+// overlap the previous kernel of the stream; it waits for that one's results
+// (griddepcontrol.wait) before it touches global memory.
+template <typename... Args>
+cudaError_t launch_dependent(void (*kern)(Args...), unsigned grid, unsigned threads, size_t smem,
+                             cudaStream_t st, Args... args) {
+  if (smem > 0) {
+    cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+    if (e != cudaSuccess) return e;
   }
-  __syncthreads();
-  for (int k = threadIdx.y; k < 32; k += blockDim.y) {
-    const int64_t c = c0 + k, r = r0 + threadIdx.x;
-    if (r < R && c < C) out[c * R + r] = tile[threadIdx.x][k];
-  }
+  cudaLaunchAttribute attr{};
+  attr.id = cudaLaunchAttributeProgrammaticStreamSerialization;
+  attr.val.programmaticStreamSerializationAllowed = 1;
+  cudaLaunchConfig_t cfg{};
+  cfg.gridDim = dim3(grid);
+  cfg.blockDim = dim3(threads);
+  cfg.dynamicSmemBytes = smem;
+  cfg.stream = st;
+  cfg.attrs = &attr;
+  cfg.numAttrs = 1;
+  return cudaLaunchKernelEx(&cfg, kern, args...);
+}
+
+template <bool AMN, bool BMN, int OP>
+cudaError_t launch_gemm(const void* A, int64_t M, const void* B, int N, int64_t K, int slices,
+                        const MlpEpi& epi, int* err, cudaStream_t st) {
+  if (M <= 0 || N <= 0) return cudaSuccess;
+  Job j;
+  if (!make_job(j, AMN, A, M, BMN, B, N, K, slices, epi)) return cudaErrorInvalidValue;
+  return launch_dependent(gemm_bf16_kernel<AMN, BMN, OP>, (unsigned)(j.gx * j.gy * j.gz), GM_THREADS,
+                          GM_SMEM, st, j, err);
+}
+
+// Slices of a weight gradient's contraction: few output tiles, a long contraction,
+// so split it until the tiles fill `ctas`, at least two stages per slice.
+int weight_slices(int64_t B, int Nout, int Nin, int ctas) {
+  const int64_t tiles = (int64_t)((Nout + GM_TILE - 1) / GM_TILE) * ((Nin + GM_TILE - 1) / GM_TILE);
+  const int64_t nk = B / GM_BK;
+  int64_t per = (tiles * nk + ctas - 1) / ctas;
+  if (per < 2) per = 2;
+  return (int)((nk + per - 1) / per);
+}
+
+// rows of Y (FP32, p wide; selected by idx when given) -> BF16 rows pk wide, and
+// their support slots (-1 padded to 16) when sup is given; and clears zero_len
+// floats at zero (the gradients of the step).
+__global__ void gather_rows_kernel(const float* __restrict__ Y, int p, int pk,
+                                   const int64_t* __restrict__ idx, int64_t B,
+                                   const int32_t* __restrict__ sup_in, int s,
+                                   __nv_bfloat16* __restrict__ X, int32_t* __restrict__ sup_out,
+                                   float4* __restrict__ zero, int64_t zero_len4) {
+  asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
+  asm volatile("griddepcontrol.wait;" ::: "memory");
+  const int64_t e = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
+  for (int64_t q = e; q < zero_len4; q += (int64_t)gridDim.x * blockDim.x)
+    zero[q] = make_float4(0.f, 0.f, 0.f, 0.f);
+  if (e >= B * pk) return;
+  const int64_t b = e / pk;
+  const int c = (int)(e - b * pk);
+  const int64_t r = idx ? idx[b] : b;
+  X[e] = __float2bfloat16_rn(c < p ? Y[r * p + c] : 0.f);
+  if (sup_in && c < 16) sup_out[b * 16 + c] = c < s ? sup_in[r * s + c] : -1;
 }
 
 __global__ void f32_to_bf16_kernel(const float* __restrict__ in, int64_t count,
                                    __nv_bfloat16* __restrict__ out) {
   const int64_t e = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
   if (e < count) out[e] = __float2bfloat16_rn(in[e]);
-}
-
-// dz = (sigmoid(z) - t) / B as BF16, t = 1 on the signal's support; the BCE
-// loss sum(softplus(z) - t z) / B is accumulated into *loss (double).
-__global__ void bce_grad_kernel(const float* __restrict__ z, int64_t B, int n,
-                                const int32_t* __restrict__ sup, int s, __nv_bfloat16* __restrict__ dz,
-                                double* __restrict__ loss) {
-  __shared__ double red[8];
-  const int64_t e = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
-  double l = 0.0;
-  if (e < B * n) {
-    const int64_t b = e / n;
-    const int j = (int)(e - b * n);
-    float t = 0.f;
-    for (int q = 0; q < s; ++q)
-      if (sup[b * s + q] == j) t = 1.f;
-    const float zz = z[e];
-    const float sg = 1.f / (1.f + expf(-zz));
-    dz[e] = __float2bfloat16_rn((sg - t) / (float)B);
-    const float sp = zz > 0.f ? zz + log1pf(expf(-zz)) : log1pf(expf(zz));
-    l = (double)(sp - t * zz) / (double)B;
-  }
-#pragma unroll
-  for (int o = 16; o > 0; o >>= 1) l += __shfl_xor_sync(0xffffffffu, l, o);
-  if ((threadIdx.x & 31) == 0) red[threadIdx.x >> 5] = l;
-  __syncthreads();
-  if (threadIdx.x == 0) {
-    double t = 0.0;
-    for (int w = 0; w < (int)(blockDim.x >> 5); ++w) t += red[w];
-    atomicAdd(loss, t);
-  }
-}
-
-// out[c] += sum over a 256-row slice of in[r][c] (BF16 rows, FP32 sums); the
-// caller zeroes out.  grid = (column blocks, row slices).
-__global__ void colsum_bf16_kernel(const __nv_bfloat16* __restrict__ in, int64_t R, int C,
-                                   float* __restrict__ out) {
-  const int c = blockIdx.x * blockDim.x + threadIdx.x;
-  if (c >= C) return;
-  const int64_t r0 = (int64_t)blockIdx.y * 256;
-  const int64_t r1 = r0 + 256 < R ? r0 + 256 : R;
-  float acc = 0.f;
-  for (int64_t r = r0; r < r1; ++r) acc += __bfloat162float(in[r * C + c]);
-  atomicAdd(out + c, acc);
 }
 
 // Adam (Kingma & Ba) on FP32 master weights; refreshes the BF16 copy.
@@ -377,67 +522,50 @@ __global__ void topk_kernel(const T* __restrict__ z, int64_t ld, int64_t m, int 
 
 bool mlp_gemm_supported() { return encode_fn() != nullptr; }
 
-cudaError_t mlp_gemm(const void* A, int64_t M, const void* B, int N, int K, int op, const float* bias,
-                     const float* aux, int64_t ldaux, float* out_f32, void* out_bf16, int64_t ldc,
-                     int* err, cudaStream_t st) {
-  if (M <= 0 || N <= 0) return cudaSuccess;
-  if (K % GM_BK != 0) return cudaErrorInvalidValue;
-  CUtensorMap ma, mb;
-  if (!map_bf16(&ma, A, M, K, GM_TILE_M) || !map_bf16(&mb, B, N, K, GM_BLOCK_N))
-    return cudaErrorInvalidValue;
-  const size_t smem = 1024 + GM_STAGES * (GM_A_BYTES + GM_B_BYTES) + 128;
-  cudaError_t e =
-      cudaFuncSetAttribute(gemm_bf16_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
-  if (e != cudaSuccess) return e;
-  Epi epi{op, bias, aux, ldaux, out_f32, (__nv_bfloat16*)out_bf16, ldc};
-  const unsigned gx = (unsigned)((M + GM_TILE_M - 1) / GM_TILE_M);
-  const unsigned gy = (unsigned)((N + GM_BLOCK_N - 1) / GM_BLOCK_N);
-  // small output grids with long K (weight gradients) split K across CTAs and
-  // accumulate FP32 atomically (bias added by a separate pass is not needed:
-  // those products have no bias)
-  unsigned gz = 1;
-  const int nk = K / GM_BK;
-  if (op == MLP_EPI_F32 && !bias) {
-    const unsigned want = (unsigned)(2 * num_sms()) / (gx * gy);
-    gz = want < 1 ? 1 : want;
-    if (gz > (unsigned)nk / 2) gz = nk / 2 > 0 ? (unsigned)(nk / 2) : 1;
+cudaError_t mlp_forward(const void* A, int64_t M, const void* W, int N, int K, int op,
+                        const MlpEpi& epi, int* err, cudaStream_t st) {
+  switch (op) {
+    case MLP_EPI_GELU_FWD: return launch_gemm<false, false, MLP_EPI_GELU_FWD>(A, M, W, N, K, 1, epi, err, st);
+    case MLP_EPI_LOGITS: return launch_gemm<false, false, MLP_EPI_LOGITS>(A, M, W, N, K, 1, epi, err, st);
+    case MLP_EPI_BCE: return launch_gemm<false, false, MLP_EPI_BCE>(A, M, W, N, K, 1, epi, err, st);
+    default: return cudaErrorInvalidValue;
   }
-  if (gz > 1) {
-    e = cudaMemsetAsync(out_f32, 0, sizeof(float) * (size_t)M * ldc, st);
-    if (e != cudaSuccess) return e;
-  }
-  gemm_bf16_kernel<<<dim3(gx, gy, gz), GM_THREADS, smem, st>>>(ma, mb, M, N, K, epi, err);
-  return cudaGetLastError();
 }
 
-cudaError_t mlp_transpose(const void* in, int64_t R, int64_t C, void* out, cudaStream_t st) {
-  if (R <= 0 || C <= 0) return cudaSuccess;
-  dim3 grid((unsigned)((C + 31) / 32), (unsigned)((R + 31) / 32));
-  transpose_bf16_kernel<<<grid, dim3(32, 8), 0, st>>>((const __nv_bfloat16*)in, R, C,
-                                                       (__nv_bfloat16*)out);
-  return cudaGetLastError();
+cudaError_t mlp_backward(const void* dY, int64_t B, const void* W, int Nout, int Nin, const MlpEpi& epi,
+                         const void* X, float* dW, int* err, cudaStream_t st) {
+  Job d, w;
+  MlpEpi ew{};
+  ew.out_f32 = dW;
+  ew.ldc = Nin;
+  if (!make_job(d, false, dY, B, true, W, Nin, Nout, 1, epi)) return cudaErrorInvalidValue;
+  int room = 2 * num_sms() - d.gx * d.gy;  // CTAs beside the input gradient's (at least one per SM)
+  if (room < num_sms()) room = num_sms();
+  if (!make_job(w, true, dY, Nout, true, X, Nin, B, weight_slices(B, Nout, Nin, room), ew))
+    return cudaErrorInvalidValue;
+  return launch_dependent(gemm_backward_kernel, (unsigned)(d.gx * d.gy + w.gx * w.gy * w.gz), GM_THREADS,
+                          GM_SMEM, st, d, w, err);
+}
+
+cudaError_t mlp_backward_weight(const void* dY, const void* X, int64_t B, int Nout, int Nin, float* dW,
+                                int* err, cudaStream_t st) {
+  MlpEpi epi{};
+  epi.out_f32 = dW;
+  epi.ldc = Nin;
+  return launch_gemm<true, true, MLP_EPI_RED>(dY, Nout, X, Nin, B,
+                                              weight_slices(B, Nout, Nin, num_sms()), epi, err, st);
+}
+
+cudaError_t mlp_gather(const float* Y, int p, int pk, const int64_t* idx, int64_t B, const int32_t* sup_in,
+                       int s, void* X, int32_t* sup_out, float* zero, int64_t zero_len, cudaStream_t st) {
+  const int64_t tot = B * pk;
+  return launch_dependent(gather_rows_kernel, (unsigned)((tot + 255) / 256), 256u, (size_t)0, st, Y, p, pk,
+                          idx, B, sup_in, s, (__nv_bfloat16*)X, sup_out, (float4*)zero, zero_len / 4);
 }
 
 cudaError_t mlp_to_bf16(const float* in, int64_t count, void* out, cudaStream_t st) {
   if (count <= 0) return cudaSuccess;
   f32_to_bf16_kernel<<<(unsigned)((count + 255) / 256), 256, 0, st>>>(in, count, (__nv_bfloat16*)out);
-  return cudaGetLastError();
-}
-
-cudaError_t mlp_bce_grad(const float* z, int64_t B, int n, const int32_t* sup, int s, void* dz,
-                         double* loss, cudaStream_t st) {
-  const int64_t tot = B * n;
-  if (tot <= 0) return cudaSuccess;
-  bce_grad_kernel<<<(unsigned)((tot + 255) / 256), 256, 0, st>>>(z, B, n, sup, s,
-                                                                 (__nv_bfloat16*)dz, loss);
-  return cudaGetLastError();
-}
-
-cudaError_t mlp_colsum(const void* in, int64_t R, int C, float* out, cudaStream_t st) {
-  cudaError_t e = cudaMemsetAsync(out, 0, sizeof(float) * (size_t)C, st);
-  if (e != cudaSuccess) return e;
-  dim3 grid((unsigned)((C + 127) / 128), (unsigned)((R + 255) / 256));
-  colsum_bf16_kernel<<<grid, 128, 0, st>>>((const __nv_bfloat16*)in, R, C, out);
   return cudaGetLastError();
 }
 
