@@ -285,7 +285,7 @@ bool tc_ok(dl_ctx* c, const float* Y, const float* D) {
 }
 
 cudaError_t enq_gram(dl_ctx* c, const float* D, bool tc) {
-  if (!tc) return dlk::gemm_nt_simt(D, c->n, D, c->n, c->p, c->G, c->n, c->st);
+  if (!tc) return dlk::gram_simt(D, c->n, c->p, c->G, c->st);  // (the same sums as gemm_nt_simt)
   cudaError_t e = dlk::split_tf32(D, (int64_t)c->n * c->p, c->Dhi, c->Dlo, c->st);
   if (e != cudaSuccess) return e;
   return dlk::corr_tf32x3(D, c->n, c->Dhi, c->Dlo, c->n, c->p, c->G, c->n, c->err, c->st);
@@ -416,6 +416,11 @@ cudaError_t enq_omp(dl_ctx* c, const float* Y, int64_t m, const float* D, int s)
                               c->err, c->st);
     if (e != cudaSuccess) return e;
     c->omp_kernels[0] = 2 /* split, products */ + 2 /* OMP, FP64 re-solve */;
+  } else if (!tc && !learned && !lp_ok(c)) {  // the same on the CUDA cores
+    mark(c, 1);
+    e = dlk::gemm_nt_simt_pair(Y, m, c->A0, c->lda, D, c->n, c->G, c->n, D, c->n, c->p, c->st);
+    if (e != cudaSuccess) return e;
+    c->omp_kernels[0] = 1 /* products */ + 2 /* OMP, FP64 re-solve */;
   } else {
     if ((e = enq_gram(c, D, tc)) != cudaSuccess) return e;
     mark(c, 1);

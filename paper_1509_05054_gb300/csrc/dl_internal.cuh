@@ -28,6 +28,10 @@ constexpr float kGapTol = 4e-6f;
 // C[i*ldc + j] = sum_r A[i*p + r] * B[j*p + r]  for i < rows_a, j < rows_b (FP32, CUDA cores)
 cudaError_t gemm_nt_simt(const float* A, int64_t rows_a, const float* B, int rows_b, int p, float* C,
                          int64_t ldc, cudaStream_t st);
+// Two products with the same B in one launch: C0 = A0 B^T and C1 = A1 B^T (A1 may be null).
+cudaError_t gemm_nt_simt_pair(const float* A0, int64_t rows0, float* C0, int64_t ldc0, const float* A1,
+                              int64_t rows1, float* C1, int64_t ldc1, const float* B, int rows_b, int p,
+                              cudaStream_t st);
 // G = D D^T (n x n, exactly symmetric), FP32 on the CUDA cores in one short launch.
 cudaError_t gram_simt(const float* D, int n, int p, float* G, cudaStream_t st);
 
