@@ -57,7 +57,7 @@ struct dl_ctx {
   int64_t lda = 0;  // row stride of the correlation matrix A0 (floats)
   // workspace
   float* G = nullptr;
-  float* A0 = nullptr;
+  float* A0 = nullptr;   // m_max x max(lda, p): alpha0, then the errors of the atom update
   int jau_kernels = 5;   // kernel launches of the last enqueued JAU update
   int ntilde = 0;        // group size of the atom update (0 or n: all atoms at once)
   int rule = DL_RULE_AKSVD;  // atom update rule
@@ -461,9 +461,13 @@ int group_size(dl_ctx* c) { return c->ntilde > 0 && c->ntilde < c->n ? c->ntilde
 cudaError_t enq_jau(dl_ctx* c, const float* Y, int64_t m, float* D, int s, const int64_t* colptr,
                     int32_t* rowidx_out, float* val_out, cudaEvent_t join) {
   c->jw.det = c->deterministic && dlk::jau_det_supported(c->p, c->n, s, Y, D);
+  // the errors go where the coding pass kept alpha0, which nothing reads any more
+  const bool plain = group_size(c) == c->n && c->rule != DL_RULE_NSGK && !c->jw.det && m > 0;
+  c->jw.E = plain && dlk::jau_plain_supported(m, c->p, c->n, s, Y, D) ? c->A0 : nullptr;
   c->jw.nb_accum = c->jw.det ? (int)dlk::jau_det_ranges(m, c->p, c->n, s)
+                   : c->jw.E ? dlk::jau_plain_blocks(c->p)
                              : dlk::jau_accum_blocks(c->p, c->n, c->cfg_acc_mult);
-  c->jw.nb_row = dlk::jau_row_blocks(c->cfg_row_per_sm);
+  c->jw.nb_row = c->jw.E ? dlk::jau_plain_row_blocks(c->p) : dlk::jau_row_blocks(c->cfg_row_per_sm);
   const int nt = group_size(c);
   const int ngroups = (c->n + nt - 1) / nt;
   const bool nsgk = c->rule == DL_RULE_NSGK;
@@ -478,7 +482,7 @@ cudaError_t enq_jau(dl_ctx* c, const float* Y, int64_t m, float* D, int s, const
                                     cudaMemcpyDeviceToDevice, c->st)) != cudaSuccess)
     return e0;
   // (groups need the float4 passes; the entry points check this before enqueuing)
-  c->jau_kernels = (dlk::jau_launches(c->p, Y, D) - 1) * ngroups + 1;
+  c->jau_kernels = (dlk::jau_launches(c->p, Y, D) - 1) * ngroups + 1 + (c->jw.E ? 1 : 0);
   mark(c, 4);
   cudaError_t e = cudaSuccess;
   for (int a0 = 0; a0 < c->n; a0 += nt) {
@@ -849,7 +853,7 @@ int dl_init(dl_ctx** out, int p, int n, int64_t m_max, int s_max, int precision,
   size_t nslices = dlk::jau_accum_smem(p, n) > 0 ? (size_t)c->jw.nb_accum : 1;
   if (nslices < (size_t)dlk::kUCopies) nslices = dlk::kUCopies;
   if (nslices < (size_t)nbd) nslices = (size_t)nbd;
-  bool ok = dalloc(&c->G, (size_t)n * n) && dalloc(&c->A0, mm * c->lda) &&
+  bool ok = dalloc(&c->G, (size_t)n * n) && dalloc(&c->A0, mm * std::max<int64_t>(c->lda, p)) &&
             dalloc(&c->sidx, mm * s_max) && dalloc(&c->sval, mm * s_max) &&
             dalloc(&c->scnt, mm) && dalloc(&c->bsum, (size_t)dlk::scan_blocks(m_max) + 1) &&
             dalloc(&c->err, 1) && dalloc(&c->iter, 1) && dalloc(&c->jw.Upart, nslices * ulen) &&

@@ -223,6 +223,9 @@ struct JauWork {
   // pass A in its deterministic form (jau_det_supported): nb_accum ranges of signals,
   // one slice of Upart each
   bool det = false;
+  // the plain case (jau_plain_supported, nb_accum = jau_plain_blocks): the errors
+  // y - D x of all signals (m x p), written by pass A and read by pass B; null otherwise
+  float* E = nullptr;
 };
 // Grid sizes: mult selects 1x/2x the base CTA count of the accumulation pass
 // and 2/4/8 CTAs per SM for the row pass; *_max give the partial-buffer sizes.
@@ -243,6 +246,10 @@ bool jau_vec4(int p, const float* Y, const float* D);
 // n <= 1024, s <= 16, a range of signals per CTA in shared memory); its CTA count.
 bool jau_det_supported(int p, int n, int s, const float* Y, const float* D);
 int64_t jau_det_ranges(int64_t m, int p, int n, int s);
+bool jau_plain_supported(int64_t m, int p, int n, int s, const float* Y, const float* D);
+int jau_plain_min();  // fewest signals
+int jau_plain_blocks(int p);
+int jau_plain_row_blocks(int p);
 int jau_launches(int p, const float* Y, const float* D);
 
 cudaError_t jau_accumulate(const float* Y, int p, int64_t m, const float* D, int n, int s,

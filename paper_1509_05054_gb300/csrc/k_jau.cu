@@ -15,6 +15,7 @@
 // they fit).  The copies are summed in a fixed order.  The energy partial sums are reduced in a
 // fixed order.
 #include "dl_internal.cuh"
+#include "tc_ptx.cuh"
 
 #include <math.h>
 
@@ -279,6 +280,376 @@ __global__ void __launch_bounds__(ACC4_THREADS, 4) accum4_kernel(
     epart[2 * blockIdx.x] = see;
     epart[2 * blockIdx.x + 1] = syy;
   }
+}
+
+// ---- The plain case: errors, bucketed sums, rows -------------------------------
+// All atoms at once (no groups, no P-NSGK), float4 rows.  What bounds accum4_kernel
+// is the L2's reduction rate: s rows of p floats per signal, 205 MB of vector
+// reductions at p = 64, n = 512, s = 8, m = 1e5 (44.9 us), and what bounds
+// rows4_kernel is issuing about 1,000 instructions per four signals (33.7 us).
+// Three passes instead:
+//   errors_kernel  E = Y - D X, stored; no shared memory, so that L1 holds the
+//                  atoms (gathered from L2 they cost twice as much);
+//   sums_kernel    U = E X^T and r: a CTA takes a tile of E into shared memory,
+//                  buckets the tile's (signal, x) pairs by atom (a counting sort: the
+//                  shared-memory counter of the atom gives the pair's rank), and
+//                  sums runs of equal atoms in registers; U in L2 gets one row
+//                  per atom and tile (plus one per share of the pairs);
+//   rows_kernel    x' and the final error from E and the rows of D'.
+// The eight lanes of a signal take four slots at a time without branches, so that
+// eight 16-byte gathers per lane are in flight; the four dot products of a group
+// are summed together by halving exchanges (4 shuffles instead of 12).
+// Measured at the size above: 16.9, 18.2 and 17.9 us.
+constexpr int EP_THREADS = 256;
+
+// Two packed multiply-adds: c + a b.
+__device__ __forceinline__ float4 f4_fma2(float a, float4 b, float4 c) {
+  const float2 lo = __ffma2_rn(make_float2(a, a), make_float2(b.x, b.y), make_float2(c.x, c.y));
+  const float2 hi = __ffma2_rn(make_float2(a, a), make_float2(b.z, b.w), make_float2(c.z, c.w));
+  return make_float4(lo.x, lo.y, hi.x, hi.y);
+}
+__device__ __forceinline__ float f4_sum(float4 v) { return (v.x + v.y) + (v.z + v.w); }
+
+// Lane g's vector q of a row of pv vectors at base (valid when g + 8 q < pv).
+template <int RV, bool FULLP>
+__device__ __forceinline__ void load_row(float4 (&r)[RV], const float4* base, int g, int pv, bool on) {
+#pragma unroll
+  for (int q = 0; q < RV; ++q)
+    r[q] = on && (FULLP || g + 8 * q < pv) ? __ldg(base + g + 8 * q) : make_float4(0.f, 0.f, 0.f, 0.f);
+}
+
+// The same of a row that is read once: not kept in L1, which is left to the atoms.
+__device__ __forceinline__ float4 ld_once(const float4* a) {
+  float4 v;
+  asm("ld.global.nc.L1::no_allocate.v4.f32 {%0, %1, %2, %3}, [%4];"
+      : "=f"(v.x), "=f"(v.y), "=f"(v.z), "=f"(v.w)
+      : "l"(a));
+  return v;
+}
+template <int RV, bool FULLP>
+__device__ __forceinline__ void load_once(float4 (&r)[RV], const float4* base, int g, int pv, bool on) {
+#pragma unroll
+  for (int q = 0; q < RV; ++q)
+    r[q] = on && (FULLP || g + 8 * q < pv) ? ld_once(base + g + 8 * q) : make_float4(0.f, 0.f, 0.f, 0.f);
+}
+
+// A signal's slots over its eight lanes: lane g holds slots g and g + 8.
+struct Slots {
+  int c, j0, j1;
+  float x0, x1;
+};
+__device__ __forceinline__ Slots load_slots(int64_t i, bool live, int g, int s, const int32_t* __restrict__ idx,
+                                            const float* __restrict__ val, const int32_t* __restrict__ cnt) {
+  Slots q;
+  q.c = live ? cnt[i] : 0;
+  const bool a = live && g < s, b = live && g + 8 < s;  // (unused slots: atom -1, masked by the count)
+  q.j0 = a ? idx[i * s + g] : -1;
+  q.x0 = a ? val[i * s + g] : 0.f;
+  q.j1 = b ? idx[i * s + g + 8] : -1;
+  q.x1 = b ? val[i * s + g + 8] : 0.f;
+  return q;
+}
+
+template <int RV, bool FULLP>
+__global__ void __launch_bounds__(EP_THREADS, RV <= 2 ? 4 : 3) errors_kernel(
+    const float* __restrict__ Y, int p, int64_t m, const float* __restrict__ D, int s,
+    const int32_t* __restrict__ idx, const float* __restrict__ val, const int32_t* __restrict__ cnt,
+    float* __restrict__ E, double* __restrict__ epart, int* __restrict__ err) {
+  __shared__ double red[EP_THREADS / 32];
+  const int lane = threadIdx.x & 31, g = lane & 7, gbase = lane & ~7;
+  const int pv = p >> 2;
+  const float4* __restrict__ D4 = (const float4*)D;
+  float ee = 0.f, yy = 0.f;
+  const int64_t groups = (int64_t)gridDim.x * (EP_THREADS / 8);
+  const int64_t trips = (m + groups - 1) / groups;
+  int64_t i = (int64_t)blockIdx.x * (EP_THREADS / 8) + (threadIdx.x >> 3);
+  Slots next = load_slots(i, i < m, g, s, idx, val, cnt);
+  for (int64_t k = 0; k < trips; ++k, i += groups) {
+    const bool live = i < m;
+    const Slots sl = next;  // (loaded a trip ahead: the gathers start at once)
+    float4 e[RV];
+    load_once<RV, FULLP>(e, (const float4*)Y + (live ? i : 0) * pv, g, pv, live);
+    next = load_slots(i + groups, i + groups < m, g, s, idx, val, cnt);
+    const int c = sl.c, o0 = sl.j0 * pv, o1 = sl.j1 * pv;  // row offsets in vectors
+    const float x0 = sl.x0, x1 = sl.x1;
+    const int cmax = __reduce_max_sync(FULL, (unsigned)c);
+    for (int t0 = 0; t0 < cmax; t0 += 4) {
+      float4 d[4][RV];
+      float x[4];
+#pragma unroll
+      for (int u = 0; u < 4; ++u) {
+        const int src = gbase + ((t0 + u) & 7);
+        const int o = __shfl_sync(FULL, t0 < 8 ? o0 : o1, src);
+        x[u] = __shfl_sync(FULL, t0 < 8 ? x0 : x1, src);
+        load_row<RV, FULLP>(d[u], D4 + o, g, pv, t0 + u < c);
+      }
+      if (t0 == 0) {
+#pragma unroll
+        for (int q = 0; q < RV; ++q) yy = f4_dot(e[q], e[q], yy);
+      }
+#pragma unroll
+      for (int u = 0; u < 4; ++u)
+#pragma unroll
+        for (int q = 0; q < RV; ++q) e[q] = f4_fma2(t0 + u < c ? -x[u] : 0.f, d[u][q], e[q]);
+    }
+    if (cmax == 0) {
+#pragma unroll
+      for (int q = 0; q < RV; ++q) yy = f4_dot(e[q], e[q], yy);
+    }
+#pragma unroll
+    for (int q = 0; q < RV; ++q) {
+      ee = f4_dot(e[q], e[q], ee);
+      if (live && (FULLP || g + 8 * q < pv)) ((float4*)E)[i * pv + g + 8 * q] = e[q];
+    }
+  }
+  if (!isfinite(ee) || !isfinite(yy)) atomicOr(err, ERR_NONFINITE);
+  const double see = block_sum_d((double)ee, red);
+  const double syy = block_sum_d((double)yy, red);
+  if (threadIdx.x == 0) {
+    epart[2 * blockIdx.x] = see;
+    epart[2 * blockIdx.x + 1] = syy;
+  }
+}
+
+constexpr int SUM_THREADS = 512;
+constexpr int SUM_SHARES = SUM_THREADS / 16;     // half warps
+constexpr int SUM_KEEP = 6;                      // pairs a thread keeps in registers
+constexpr size_t SUM_SMEM = 113 * 1024;          // dynamic, two CTAs per SM
+struct SumSmem {  // byte offsets, T signals per tile (T % 4 == 0)
+  int np, sk, sx, off, rank, total;
+  __host__ __device__ SumSmem(int p, int n, int s, int T) {
+    np = (T * s + 4 * SUM_SHARES - 1) / (4 * SUM_SHARES) * (4 * SUM_SHARES);  // padded pairs
+    sk = T * p * 4;         // after the errors [T][p]: sorted pairs, atom << 16 | signal
+    sx = sk + np * 4;       // their x
+    off = sx + np * 4;      // pairs per atom, then bucket starts
+    rank = off + n * 4;     // rank of each pair in its bucket (u16; unsorted)
+    total = rank + (T * s * 2 + 15) / 16 * 16;
+  }
+};
+// Signals per tile: equal tiles for two CTAs per SM, as few per CTA as fit; at
+// least 64 where there are few signals.  0: none fits.
+int sum_tile(int64_t m, int p, int n, int s) {
+  const int64_t g = 2 * num_sms();
+  for (int64_t k = 1;; ++k) {
+    int64_t T = (m + g * k - 1) / (g * k);
+    if (T < 64) T = 64;
+    T = (T + 3) / 4 * 4;
+    if (T * s < 65536 && T < 65536 && (size_t)SumSmem(p, n, s, (int)T).total <= SUM_SMEM) return (int)T;
+    if (T == 64) return 0;
+  }
+}
+
+__global__ void __launch_bounds__(SUM_THREADS, 2) sums_kernel(
+    const float* __restrict__ E, int p, int64_t m, int T, int n, int s, const int32_t* __restrict__ idx,
+    const float* __restrict__ val, float* __restrict__ U, int* __restrict__ err) {
+  extern __shared__ __align__(128) uint8_t ssh[];
+  __shared__ int wsum[SUM_THREADS / 32];
+  __shared__ uint64_t bar;
+  const SumSmem lay(p, n, s, T);
+  const float* Es = (const float*)ssh;
+  uint32_t* sk = (uint32_t*)(ssh + lay.sk);
+  float* sx = (float*)(ssh + lay.sx);
+  int* off = (int*)(ssh + lay.off);
+  uint16_t* rank = (uint16_t*)(ssh + lay.rank);
+  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+  const int pv = p >> 2;
+  float* __restrict__ Uc = U + (size_t)(blockIdx.x % kUCopies) * jau_ulen(p, n);
+  if (threadIdx.x == 0) {
+    tc::mbar_init(&bar, 1);
+    asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
+  }
+  const int64_t ntiles = (m + T - 1) / T;
+  uint32_t phase = 0;
+  for (int64_t tile = blockIdx.x; tile < ntiles; tile += gridDim.x, phase ^= 1) {
+    const int64_t lo = tile * T;
+    const int nr = (int)(m - lo < T ? m - lo : T);
+    const int npair = nr * s;
+    __syncthreads();  // the previous tile has been summed
+    if (threadIdx.x == 0) {  // the tile's errors, one bulk copy (rows are contiguous; p % 4 == 0)
+      const uint32_t bytes = (uint32_t)nr * (uint32_t)p * 4u;
+      asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
+      tc::mbar_expect_tx(&bar, bytes);
+      asm volatile(
+          "cp.async.bulk.shared::cluster.global.mbarrier::complete_tx::bytes [%0], [%1], %2, [%3];" ::"r"(
+              tc::smem_u32(ssh)),
+          "l"(E + lo * p), "r"(bytes), "r"(tc::smem_u32(&bar))
+          : "memory");
+    }
+    for (int a = threadIdx.x; a < n; a += SUM_THREADS) off[a] = 0;
+    __syncthreads();
+    // ---- each pair's rank in its atom's bucket (unused slots hold atom -1); a thread's
+    // first pairs stay in registers
+    int ka[SUM_KEEP], kr[SUM_KEEP];
+    float kx[SUM_KEEP];
+#pragma unroll
+    for (int u = 0; u < SUM_KEEP; ++u) {
+      const int k = threadIdx.x + u * SUM_THREADS;
+      ka[u] = k < npair ? idx[lo * s + k] : -1;
+      kx[u] = k < npair ? val[lo * s + k] : 0.f;
+    }
+#pragma unroll
+    for (int u = 0; u < SUM_KEEP; ++u) kr[u] = ka[u] >= 0 ? atomicAdd(&off[ka[u]], 1) : 0;
+    for (int k = threadIdx.x + SUM_KEEP * SUM_THREADS; k < npair; k += SUM_THREADS) {
+      const int a = idx[lo * s + k];
+      if (a >= 0) rank[k] = (uint16_t)atomicAdd(&off[a], 1);
+    }
+    __syncthreads();
+    // ---- bucket starts: exclusive scan of the counts in place, two atoms per thread (n <= 1024)
+    int np = 0;
+    {
+      const int a = 2 * threadIdx.x;
+      const int v0 = a < n ? off[a] : 0, v1 = a + 1 < n ? off[a + 1] : 0;
+      int inc = v0 + v1;
+#pragma unroll
+      for (int o = 1; o < 32; o <<= 1) {
+        const int x = __shfl_up_sync(FULL, inc, o);
+        if (lane >= o) inc += x;
+      }
+      if (lane == 31) wsum[warp] = inc;
+      __syncthreads();
+      int before = 0;
+#pragma unroll
+      for (int w = 0; w < SUM_THREADS / 32; ++w) {
+        const int x = wsum[w];
+        if (w < warp) before += x;
+        np += x;
+      }
+      const int ex = before + inc - v0 - v1;
+      if (a < n) off[a] = ex;
+      if (a + 1 < n) off[a + 1] = ex + v0;
+    }
+    const int share = (np + 4 * SUM_SHARES - 1) / (4 * SUM_SHARES) * 4;  // pairs per half warp
+    __syncthreads();
+#pragma unroll
+    for (int u = 0; u < SUM_KEEP; ++u)
+      if (ka[u] >= 0) {
+        const int pos = off[ka[u]] + kr[u];
+        sk[pos] = (uint32_t)ka[u] << 16 | (uint32_t)((threadIdx.x + u * SUM_THREADS) / s);
+        sx[pos] = kx[u];
+      }
+    for (int k = threadIdx.x + SUM_KEEP * SUM_THREADS; k < npair; k += SUM_THREADS) {
+      const int a = idx[lo * s + k];
+      if (a >= 0) {
+        const int pos = off[a] + rank[k];
+        sk[pos] = (uint32_t)a << 16 | (uint32_t)(k / s);
+        sx[pos] = val[lo * s + k];
+      }
+    }
+    for (int k = np + threadIdx.x; k < share * SUM_SHARES; k += SUM_THREADS) {  // no atom
+      sk[k] = 0xffff0000u;
+      sx[k] = 0.f;
+    }
+    const bool ok = tc::mbar_wait(&bar, phase);
+    if (!ok && threadIdx.x == 0) atomicOr(err, ERR_TIMEOUT);
+    if (!__syncthreads_and(ok)) break;
+    // ---- sums over runs of equal atoms: half a warp takes an equal share of the pairs, 16 lanes a row
+    const int hw = threadIdx.x >> 4, l16 = threadIdx.x & 15;
+    const int k1 = (hw + 1) * share;
+    for (int q0 = 0; q0 < pv; q0 += 16) {  // (a second round of vectors for p > 64)
+      const bool on = q0 + l16 < pv;
+      const float* col = Es + 4 * (on ? q0 + l16 : 0);
+      float4 acc = make_float4(0.f, 0.f, 0.f, 0.f);
+      float rx = 0.f;
+      for (int k = hw * share; k < k1; k += 4) {
+        const uint4 K = *(const uint4*)(sk + k);
+        const float4 X = *(const float4*)(sx + k);
+        const uint32_t next = k + 4 < k1 ? sk[k + 4] >> 16 : ~0u;
+        const uint32_t at[5] = {K.x >> 16, K.y >> 16, K.z >> 16, K.w >> 16, next};
+        const float x[4] = {X.x, X.y, X.z, X.w};
+        float4 r[4];
+        r[0] = *(const float4*)(col + (K.x & 0xffffu) * p);
+        r[1] = *(const float4*)(col + (K.y & 0xffffu) * p);
+        r[2] = *(const float4*)(col + (K.z & 0xffffu) * p);
+        r[3] = *(const float4*)(col + (K.w & 0xffffu) * p);
+#pragma unroll
+        for (int h = 0; h < 4; ++h) {
+          acc = f4_fma2(x[h], r[h], acc);
+          rx = fmaf(x[h], x[h], rx);
+          if (at[h] != at[h + 1]) {  // the run ends
+            if (at[h] != 0xffffu) {
+              if (on) red_add_v4(Uc + ((size_t)at[h] * pv + q0 + l16) * 4, acc);
+              if (l16 == 0 && q0 == 0) atomicAdd(Uc + (size_t)n * p + at[h], rx);
+            }
+            acc = make_float4(0.f, 0.f, 0.f, 0.f);
+            rx = 0.f;
+          }
+        }
+      }
+    }
+  }
+}
+
+// Pass B of the plain case: x_t' = e.d'_{j_t} + c_{j_t} x_t (sgk: x_t) into the CSC
+// values, and ||y - D' x'||^2.
+template <int RV, bool FULLP>
+__global__ void __launch_bounds__(EP_THREADS, RV <= 1 ? 4 : RV == 2 ? 3 : 2) rows_plain_kernel(
+    const float* __restrict__ Y, const float* __restrict__ E, int p, int64_t m,
+    const float* __restrict__ Dn, const float* __restrict__ C, int s, const int32_t* __restrict__ idx,
+    const float* __restrict__ val, const int32_t* __restrict__ cnt, const int64_t* __restrict__ colptr,
+    float* __restrict__ csc_val, double* __restrict__ epart, int sgk) {
+  __shared__ double red[EP_THREADS / 32];
+  const int lane = threadIdx.x & 31, g = lane & 7, gbase = lane & ~7;
+  const int b2 = g >> 2 & 1, b1 = g >> 1 & 1, tau = 2 * b2 + b1;  // the slot of four this lane sums
+  const int pv = p >> 2;
+  const float4* __restrict__ N4 = (const float4*)Dn;
+  float e2 = 0.f;
+  const int64_t groups = (int64_t)gridDim.x * (EP_THREADS / 8);
+  const int64_t trips = (m + groups - 1) / groups;
+  int64_t i = (int64_t)blockIdx.x * (EP_THREADS / 8) + (threadIdx.x >> 3);
+  Slots next = load_slots(i, i < m, g, s, idx, val, cnt);
+  for (int64_t k = 0; k < trips; ++k, i += groups) {
+    const bool live = i < m;
+    const Slots sl = next;
+    float4 y[RV], e[RV];
+    load_once<RV, FULLP>(y, (const float4*)Y + (live ? i : 0) * pv, g, pv, live);
+    load_once<RV, FULLP>(e, (const float4*)E + (live ? i : 0) * pv, g, pv, live);
+    next = load_slots(i + groups, i + groups < m, g, s, idx, val, cnt);
+    const int c = sl.c, j0 = sl.j0, j1 = sl.j1;
+    const float x0 = sl.x0, x1 = sl.x1;
+    const float c0 = g < c ? __ldg(C + j0) : 0.f, c1 = g + 8 < c ? __ldg(C + j1) : 0.f;
+    const int64_t o = live ? colptr[i] : 0;
+    const int cmax = __reduce_max_sync(FULL, (unsigned)c);
+    for (int t0 = 0; t0 < cmax; t0 += 4) {
+      float4 d[4][RV];
+      float v[4];
+#pragma unroll
+      for (int u = 0; u < 4; ++u) {
+        const int jj = __shfl_sync(FULL, t0 < 8 ? j0 : j1, gbase + ((t0 + u) & 7));
+        load_row<RV, FULLP>(d[u], N4 + jj * pv, g, pv, t0 + u < c);
+      }
+#pragma unroll
+      for (int u = 0; u < 4; ++u) {
+        float2 a = make_float2(0.f, 0.f);
+#pragma unroll
+        for (int q = 0; q < RV; ++q) {
+          a = __ffma2_rn(make_float2(e[q].x, e[q].y), make_float2(d[u][q].x, d[u][q].y), a);
+          a = __ffma2_rn(make_float2(e[q].z, e[q].w), make_float2(d[u][q].z, d[u][q].w), a);
+        }
+        v[u] = a.x + a.y;
+      }
+      // four sums over eight lanes: lanes with bit 2 set keep slots 2 and 3, then bit 1 picks one
+      const float w0 = (b2 ? v[2] : v[0]) + __shfl_xor_sync(FULL, b2 ? v[0] : v[2], 4);
+      const float w1 = (b2 ? v[3] : v[1]) + __shfl_xor_sync(FULL, b2 ? v[1] : v[3], 4);
+      float dot = (b1 ? w1 : w0) + __shfl_xor_sync(FULL, b1 ? w0 : w1, 2);
+      dot += __shfl_xor_sync(FULL, dot, 1);
+      const int src = gbase + ((t0 + tau) & 7);
+      const float xo = __shfl_sync(FULL, t0 < 8 ? x0 : x1, src);
+      const float co = __shfl_sync(FULL, t0 < 8 ? c0 : c1, src);
+      const float xn = sgk ? xo : fmaf(co, xo, dot);
+      if (!(g & 1) && t0 + tau < c && csc_val) csc_val[o + t0 + tau] = xn;
+#pragma unroll
+      for (int u = 0; u < 4; ++u) {  // y - D' x' from the same rows (zero past the count)
+        float xu = __shfl_sync(FULL, xn, gbase + 4 * (u >> 1) + 2 * (u & 1));
+        if (t0 + u >= c) xu = 0.f;
+#pragma unroll
+        for (int q = 0; q < RV; ++q) y[q] = f4_fma2(-xu, d[u][q], y[q]);
+      }
+    }
+#pragma unroll
+    for (int q = 0; q < RV; ++q) e2 = f4_dot(y[q], y[q], e2);
+  }
+  const double se = block_sum_d((double)e2, red);
+  if (threadIdx.x == 0) epart[blockIdx.x] = se;
 }
 
 // ---- Pass A, deterministic form ---------------------------------------------
@@ -1031,6 +1402,19 @@ int jau_launches(int p, const float* Y, const float* D) {
 int jau_row_blocks(int per_sm) { return (per_sm == 2 || per_sm == 8 ? per_sm : 4) * num_sms(); }
 int jau_row_blocks_max() { return 8 * num_sms(); }
 
+// From one signal per resident eight lanes of the errors pass on: with fewer, all
+// passes are bound by launches, and accum4_kernel has one launch less (one
+// iteration at p = 16, n = 32, s = 3, m = 1000: 97.4 us against 99.2; p = 64,
+// n = 256, s = 6, m = 20,000: 77.5 against 75.8).
+bool jau_plain_supported(int64_t m, int p, int n, int s, const float* Y, const float* D) {
+  return m >= jau_plain_min() && jau_vec4(p, Y, D) && p <= 128 && n <= 1024 && s <= 16 &&
+         sum_tile(m, p, n, s) > 0;
+}
+int jau_plain_min() { return 32 * num_sms(); }
+// one full round of resident CTAs each (see the kernels' launch bounds)
+int jau_plain_blocks(int p) { return (p <= 64 ? 4 : 3) * num_sms(); }
+int jau_plain_row_blocks(int p) { return (p <= 32 ? 4 : p <= 64 ? 3 : 2) * num_sms(); }
+
 bool jau_det_supported(int p, int n, int s, const float* Y, const float* D) {
   return (Y || D ? jau_vec4(p, Y, D) : p % 4 == 0) && p <= 128 && n <= 1024 && s <= 16 &&
          det_range(p, n, s) >= 64;
@@ -1094,6 +1478,31 @@ cudaError_t jau_accumulate(const float* Y, int p, int64_t m, const float* D, int
     const size_t len = jau_ulen(p, n);
     cudaError_t e = cudaMemsetAsync(w.Upart, 0, sizeof(float) * len * kUCopies, st);
     if (e != cudaSuccess) return e;
+    if (w.E) {  // the plain case
+#define DL_ERRS(RV)                                                                              \
+  do {                                                                                           \
+    auto kern = p == 32 * RV ? errors_kernel<RV, true> : errors_kernel<RV, false>;               \
+    cudaFuncSetAttribute(kern, cudaFuncAttributePreferredSharedMemoryCarveout,                   \
+                         cudaSharedmemCarveoutMaxL1);                                            \
+    kern<<<w.nb_accum, EP_THREADS, 0, st>>>(Y, p, m, D, s, idx, val, cnt, w.E, w.epart_a, err);  \
+  } while (0)
+      if (p <= 32) DL_ERRS(1);
+      else if (p <= 64) DL_ERRS(2);
+      else if (p <= 96) DL_ERRS(3);
+      else DL_ERRS(4);
+#undef DL_ERRS
+      if ((e = cudaGetLastError()) != cudaSuccess) return e;
+      const int T = sum_tile(m, p, n, s);
+      const size_t smem = (size_t)SumSmem(p, n, s, T).total;
+      if ((e = cudaFuncSetAttribute(sums_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                    (int)smem)) != cudaSuccess)
+        return e;
+      const int64_t nt = (m + T - 1) / T;
+      sums_kernel<<<(unsigned)(nt < 2 * num_sms() ? nt : 2 * num_sms()), SUM_THREADS, smem, st>>>(
+          w.E, p, m, T, n, s, idx, val, w.Upart, err);
+      if ((e = cudaGetLastError()) != cudaSuccess) return e;
+      return reduce_slices(w.Upart, kUCopies, (int)len, w.U, st);
+    }
 #define DL_ACC4(RV, SM)                                                                  \
   do {                                                                                       \
     if (w.nsgk)                                                                              \
@@ -1160,6 +1569,22 @@ cudaError_t jau_rows(const float* Y, int p, int64_t m, const float* D, int n, in
 #define DL_ROWS(PL)                                                                              \
   rows_kernel<PL><<<nb, ROW_THREADS, 0, st>>>(Y, p, m, D, w.Dn, w.C, s, idx, val, cnt, colptr, \
                                               csc_rowidx, csc_val, w.epart_b, (int)w.sgk)
+  if (w.E && !csc_rowidx) {  // the plain case
+#define DL_ROWSP(RV)                                                                              \
+  do {                                                                                            \
+    auto kern = p == 32 * RV ? rows_plain_kernel<RV, true> : rows_plain_kernel<RV, false>;        \
+    cudaFuncSetAttribute(kern, cudaFuncAttributePreferredSharedMemoryCarveout,                    \
+                         cudaSharedmemCarveoutMaxL1);                                             \
+    kern<<<nb, EP_THREADS, 0, st>>>(Y, w.E, p, m, w.Dn, w.C, s, idx, val, cnt, colptr, csc_val,   \
+                                    w.epart_b, (int)w.sgk);                                       \
+  } while (0)
+    if (p <= 32) DL_ROWSP(1);
+    else if (p <= 64) DL_ROWSP(2);
+    else if (p <= 96) DL_ROWSP(3);
+    else DL_ROWSP(4);
+#undef DL_ROWSP
+    return cudaGetLastError();
+  }
   if (jau_vec4(p, Y, D)) {
 #define DL_ROWS4(RV, SM)                                                                         \
   do {                                                                                         \
