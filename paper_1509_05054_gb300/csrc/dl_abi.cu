@@ -141,7 +141,7 @@ struct dl_ctx {
   // side stream: the colptr scan overlaps the first pass of the atom update
   cudaStream_t st2 = nullptr;
   cudaEvent_t ev_fork = nullptr, ev_join = nullptr, ev_join2 = nullptr;
-  int scan_kernels = 2;  // side-stream kernels of the last iteration (colptr scan, rowidx)
+  int scan_kernels = 2;  // side-stream kernels of the last iteration (colptr, rowidx)
   // host-buffer calls: the signals arrive in chunks on the side stream
   static constexpr int kChunks = 3;
   cudaEvent_t ev_chunk[kChunks] = {};
@@ -154,7 +154,7 @@ struct dl_ctx {
 
 namespace {
 
-constexpr int kKernelsScan = 2;      // colptr scan
+constexpr int kKernelsScan = 2;      // colptr scan and entries
 
 void free_ctx(dl_ctx* c) {
   if (!c) return;
@@ -177,7 +177,7 @@ void free_ctx(dl_ctx* c) {
   if (c->st2) cudaStreamDestroy(c->st2);
   void* ptrs[] = {c->G, c->A0, c->Dhi, c->Dlo, c->Ylp, c->Ysc, c->Dlp, c->Dsc, c->rs_list,
                   c->rs_count, c->sidx, c->sval, c->scnt, c->bsum, c->err, c->iter, c->rmse,
-                  c->jw.Upart, c->jw.U, c->jw.epart_a, c->jw.epart_b, c->jw.Dn, c->jw.C,
+                  c->jw.Upart, c->jw.U, c->jw.Ucopy, c->jw.epart_a, c->jw.epart_b, c->jw.Dn, c->jw.C,
                   c->hY, c->hD, c->hcolptr, c->hrowidx, c->hval, c->pidx, c->pval, c->pcnt,
                   c->pvalid, c->D0};
   for (void* q : ptrs)
@@ -284,9 +284,11 @@ bool tc_ok(dl_ctx* c, const float* Y, const float* D) {
          dlk::corr_tc_supported(D, c->p, c->n, c->n);
 }
 
-cudaError_t enq_gram(dl_ctx* c, const float* D, bool tc) {
-  if (!tc) return dlk::gram_simt(D, c->n, c->p, c->G, c->st);  // (the same sums as gemm_nt_simt)
-  cudaError_t e = dlk::split_tf32(D, (int64_t)c->n * c->p, c->Dhi, c->Dlo, c->st);
+cudaError_t enq_gram(dl_ctx* c, const float* D, bool tc, int* zero = nullptr) {
+  // (gram_simt's sums are those of gemm_nt_simt; the first kernel of a coding pass
+  // also clears its count of listed signals)
+  if (!tc) return dlk::gram_simt(D, c->n, c->p, c->G, c->st, zero);
+  cudaError_t e = dlk::split_tf32(D, (int64_t)c->n * c->p, c->Dhi, c->Dlo, c->st, zero);
   if (e != cudaSuccess) return e;
   return dlk::corr_tf32x3(D, c->n, c->Dhi, c->Dlo, c->n, c->p, c->G, c->n, c->err, c->st);
 }
@@ -383,11 +385,11 @@ bool use_res(dl_ctx* c, const float* Y, const float* D, int s, int64_t m) {
 cudaError_t enq_omp_res(dl_ctx* c, const float* Y, int64_t m, const float* D, int s) {
   c->a0_bf16 = false;
   mark(c, 0);
-  cudaError_t e = dlk::gram_simt(D, c->n, c->p, c->G, c->st);  // G for the Cholesky rows
+  // G for the Cholesky rows; and the count of listed signals cleared
+  cudaError_t e = dlk::gram_simt(D, c->n, c->p, c->G, c->st, c->rs_count);
   if (e != cudaSuccess) return e;
   mark(c, 1);
   mark(c, 2);
-  if ((e = cudaMemsetAsync(c->rs_count, 0, sizeof(int), c->st)) != cudaSuccess) return e;
   c->last_omp = 2;
   e = dlk::omp_res(Y, m, c->p, D, c->n, c->G, s, c->sidx, c->sval, c->scnt, c->err, c->rs_list,
                    c->rs_count, (int)c->m_max, c->precision == DL_BF16, c->st);
@@ -410,7 +412,8 @@ cudaError_t enq_omp(dl_ctx* c, const float* Y, int64_t m, const float* D, int s)
   cudaError_t e;
   if (tc && !learned && !lp_ok(c)) {
     // one launch computes the Gram matrix and the correlations of all signals
-    if ((e = dlk::split_tf32(D, (int64_t)c->n * c->p, c->Dhi, c->Dlo, c->st)) != cudaSuccess) return e;
+    if ((e = dlk::split_tf32(D, (int64_t)c->n * c->p, c->Dhi, c->Dlo, c->st, c->rs_count)) != cudaSuccess)
+      return e;
     mark(c, 1);
     e = dlk::corr_tf32x3_pair(Y, m, c->A0, c->lda, D, c->n, c->G, c->n, c->Dhi, c->Dlo, c->n, c->p,
                               c->err, c->st);
@@ -418,19 +421,18 @@ cudaError_t enq_omp(dl_ctx* c, const float* Y, int64_t m, const float* D, int s)
     c->omp_kernels[0] = 2 /* split, products */ + 2 /* OMP, FP64 re-solve */;
   } else if (!tc && !learned && !lp_ok(c)) {  // the same on the CUDA cores
     mark(c, 1);
-    e = dlk::gemm_nt_simt_pair(Y, m, c->A0, c->lda, D, c->n, c->G, c->n, D, c->n, c->p, c->st);
+    e = dlk::gemm_nt_simt_pair(Y, m, c->A0, c->lda, D, c->n, c->G, c->n, D, c->n, c->p, c->st,
+                               c->rs_count);
     if (e != cudaSuccess) return e;
     c->omp_kernels[0] = 1 /* products */ + 2 /* OMP, FP64 re-solve */;
   } else {
-    if ((e = enq_gram(c, D, tc)) != cudaSuccess) return e;
+    if ((e = enq_gram(c, D, tc, c->rs_count)) != cudaSuccess) return e;
     mark(c, 1);
     if (learned) return enq_omp_learned(c, Y, m, D, s, tc);
     if ((e = enq_corr(c, Y, m, D, tc)) != cudaSuccess) return e;
     c->omp_kernels[0] = (tc ? 2 : 1) + (lp_ok(c) ? 2 : 1) + 2;
   }
   mark(c, 2);
-  e = cudaMemsetAsync(c->rs_count, 0, sizeof(int), c->st);
-  if (e != cudaSuccess) return e;
   const bool tm = c->cfg_omp_tm && !has_prop(c) && dlk::omp_tm_supported(c->n, s);
   const bool roll = c->cfg_omp_tm && dlk::omp_roll_supported(c->n, s);
   c->last_omp = tm || roll ? 1 : 0;
@@ -482,7 +484,8 @@ cudaError_t enq_jau(dl_ctx* c, const float* Y, int64_t m, float* D, int s, const
                                     cudaMemcpyDeviceToDevice, c->st)) != cudaSuccess)
     return e0;
   // (groups need the float4 passes; the entry points check this before enqueuing)
-  c->jau_kernels = (dlk::jau_launches(c->p, Y, D) - 1) * ngroups + 1 + (c->jw.E ? 1 : 0);
+  c->jw.copies = !c->jw.det && dlk::jau_vec4(c->p, Y, D);
+  c->jau_kernels = (dlk::jau_launches(c->jw) - 1) * ngroups + 1;
   mark(c, 4);
   cudaError_t e = cudaSuccess;
   for (int a0 = 0; a0 < c->n; a0 += nt) {
@@ -690,16 +693,13 @@ cudaError_t enq_iteration(dl_ctx* c, const float* Y, int64_t m, float* D, int s,
   if (e != cudaSuccess) return e;
   if ((e = cudaEventRecord(c->ev_fork, c->st)) != cudaSuccess) return e;
   if ((e = cudaStreamWaitEvent(c->st2, c->ev_fork, 0)) != cudaSuccess) return e;
-  e = dlk::counts_to_colptr(c->scnt, m, c->bsum, colptr, c->st2);
+  const bool side_rowidx = rowidx != nullptr && m > 0;
+  e = dlk::slots_to_csc(c->sidx, nullptr, c->scnt, m, s, c->bsum, colptr, side_rowidx ? rowidx : nullptr,
+                        nullptr, c->st2);
   if (e != cudaSuccess) return e;
   if ((e = cudaEventRecord(c->ev_join, c->st2)) != cudaSuccess) return e;  // the row pass's colptr
-  c->scan_kernels = 2;
-  const bool side_rowidx = rowidx != nullptr && m > 0;
+  c->scan_kernels = kKernelsScan;
   if (side_rowidx) {
-    if ((e = dlk::slots_to_csc(c->sidx, nullptr, c->scnt, m, s, colptr, rowidx, nullptr,
-                               c->st2)) != cudaSuccess)
-      return e;
-    c->scan_kernels = 3;
     if (colptr_dl && (e = cudaMemcpyAsync(colptr_dl, colptr, sizeof(int64_t) * (size_t)(m + 1),
                                           cudaMemcpyDeviceToHost, c->st2)) != cudaSuccess)
       return e;
@@ -851,13 +851,12 @@ int dl_init(dl_ctx** out, int p, int n, int64_t m_max, int s_max, int precision,
   c->jw.nb_row = dlk::jau_row_blocks_max();
   const size_t ulen = dlk::jau_ulen(p, n);
   size_t nslices = dlk::jau_accum_smem(p, n) > 0 ? (size_t)c->jw.nb_accum : 1;
-  if (nslices < (size_t)dlk::kUCopies) nslices = dlk::kUCopies;
   if (nslices < (size_t)nbd) nslices = (size_t)nbd;
   bool ok = dalloc(&c->G, (size_t)n * n) && dalloc(&c->A0, mm * std::max<int64_t>(c->lda, p)) &&
             dalloc(&c->sidx, mm * s_max) && dalloc(&c->sval, mm * s_max) &&
-            dalloc(&c->scnt, mm) && dalloc(&c->bsum, (size_t)dlk::scan_blocks(m_max) + 1) &&
+            dalloc(&c->scnt, mm) && dalloc(&c->bsum, (size_t)2048) &&
             dalloc(&c->err, 1) && dalloc(&c->iter, 1) && dalloc(&c->jw.Upart, nslices * ulen) &&
-            dalloc(&c->jw.U, ulen) && dalloc(&c->jw.epart_a, (size_t)2 * c->jw.nb_accum) &&
+            dalloc(&c->jw.U, ulen) && dalloc(&c->jw.Ucopy, ulen * dlk::kUCopies) && dalloc(&c->jw.epart_a, (size_t)2 * c->jw.nb_accum) &&
             dalloc(&c->jw.epart_b, (size_t)c->jw.nb_row) && dalloc(&c->jw.Dn, (size_t)n * p) &&
             dalloc(&c->jw.C, (size_t)n) && dalloc(&c->Dhi, (size_t)n * p) &&
             dalloc(&c->Dlo, (size_t)n * p) && dalloc(&c->rs_list, mm) && dalloc(&c->rs_count, 1);
@@ -1056,9 +1055,8 @@ int omp_code(dl_ctx* c, const float* Y, int64_t m, const float* D, int s, int64_
   if (needs_y_conversion(c, dY)) c->launches += 1;
   c->learned_now = false;
   DL_CHECK(enq_omp(c, dY, m, dD, s));
-  DL_CHECK(dlk::counts_to_colptr(c->scnt, m, c->bsum, dcp, c->st));
-  DL_CHECK(dlk::slots_to_csc(c->sidx, c->sval, c->scnt, m, s, dcp, dri, dv, c->st));
-  c->launches += c->omp_kernels[0] + kKernelsScan + 1;
+  DL_CHECK(dlk::slots_to_csc(c->sidx, c->sval, c->scnt, m, s, c->bsum, dcp, dri, dv, c->st));
+  c->launches += c->omp_kernels[0] + kKernelsScan;
   if (kind == 0) {
     // all s*m entries (the caller's capacity), so no synchronisation is needed to learn nnz;
     // entries past colptr[m] are unspecified

@@ -31,14 +31,16 @@ cudaError_t gemm_nt_simt(const float* A, int64_t rows_a, const float* B, int row
 // Two products with the same B in one launch: C0 = A0 B^T and C1 = A1 B^T (A1 may be null).
 cudaError_t gemm_nt_simt_pair(const float* A0, int64_t rows0, float* C0, int64_t ldc0, const float* A1,
                               int64_t rows1, float* C1, int64_t ldc1, const float* B, int rows_b, int p,
-                              cudaStream_t st);
+                              cudaStream_t st, int* zero = nullptr);
 // G = D D^T (n x n, exactly symmetric), FP32 on the CUDA cores in one short launch.
-cudaError_t gram_simt(const float* D, int n, int p, float* G, cudaStream_t st);
+// zero: an int to clear (or null).
+cudaError_t gram_simt(const float* D, int n, int p, float* G, cudaStream_t st, int* zero = nullptr);
 
 // FP32-accurate C = A B^T on tcgen05 tensor cores (split TF32, see k_corr_tc.cu).
 // B is given pre-split (B = Bhi + Blo).  Requires corr_tc_supported().
 bool corr_tc_supported(const float* A, int p, int n, int64_t ldc);
-cudaError_t split_tf32(const float* B, int64_t count, float* hi, float* lo, cudaStream_t st);
+cudaError_t split_tf32(const float* B, int64_t count, float* hi, float* lo, cudaStream_t st,
+                       int* zero = nullptr);
 cudaError_t corr_tf32x3(const float* A, int64_t rows_a, const float* Bhi, const float* Blo, int n,
                         int p, float* C, int64_t ldc, int* err, cudaStream_t st);
 // Two products with the same B in one launch: C0 = A0 B^T and C1 = A1 B^T (A1 may be null).
@@ -199,6 +201,8 @@ bool omp_supported(int n, int s);
 struct JauWork {
   float* Upart;     // [nb_accum][n*p + n] per-CTA partial U = E X^T and r = row energies
   float* U;         // [n*p + n] reduced
+  float* Ucopy;     // kUCopies copies of U and r (jau_ulen floats each)
+  bool copies;      // pass A adds to Ucopy (float4 rows, not deterministic), not to Upart
   double* epart_a;  // [nb_accum][2]  (||E||^2, ||Y||^2) partials
   double* epart_b;  // [nb_row]       ||Y - D'X'||^2 partials
   float* Dn;        // [n*p] updated atoms
@@ -250,7 +254,7 @@ bool jau_plain_supported(int64_t m, int p, int n, int s, const float* Y, const f
 int jau_plain_min();  // fewest signals
 int jau_plain_blocks(int p);
 int jau_plain_row_blocks(int p);
-int jau_launches(int p, const float* Y, const float* D);
+int jau_launches(const JauWork& w);
 
 cudaError_t jau_accumulate(const float* Y, int p, int64_t m, const float* D, int n, int s,
                            const int32_t* idx, const float* val, const int32_t* cnt,
@@ -266,12 +270,10 @@ cudaError_t jau_finalize(const JauWork& w, double* rmse_out, int* iter, float* D
                          cudaStream_t st);
 
 // ---- CSC <-> slots --------------------------------------------------------------
-int64_t scan_blocks(int64_t m);
-cudaError_t counts_to_colptr(const int32_t* cnt, int64_t m, int64_t* bsum, int64_t* colptr,
-                             cudaStream_t st);
-cudaError_t slots_to_csc(const int32_t* idx, const float* val, const int32_t* cnt, int64_t m,
-                         int s, const int64_t* colptr, int32_t* rowidx, float* cval,
-                         cudaStream_t st);
+int64_t scan_blocks(int64_t m);  // values of bsum (at most 2048)
+// colptr and, when rowidx is given, the entries (values when cval is given too).
+cudaError_t slots_to_csc(const int32_t* idx, const float* val, const int32_t* cnt, int64_t m, int s,
+                         int64_t* bsum, int64_t* colptr, int32_t* rowidx, float* cval, cudaStream_t st);
 cudaError_t csc_to_slots(const int64_t* colptr, const int32_t* rowidx, const float* cval,
                          int64_t m, int n, int s, int32_t* idx, float* val, int32_t* cnt,
                          int* err, cudaStream_t st);

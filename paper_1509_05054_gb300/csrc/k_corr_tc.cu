@@ -260,9 +260,10 @@ __global__ void __launch_bounds__(WS_THREADS, 1)
   if (threadIdx.x == 0 && *fail) atomicOr(err, ERR_TIMEOUT);
 }
 
-// Split B into TF32 head and tail (row-major, same layout as B).
+// Split B into TF32 head and tail (row-major, same layout as B); clears *zero if given.
 __global__ void split_kernel(const float* __restrict__ B, int64_t count, float* __restrict__ hi,
-                             float* __restrict__ lo) {
+                             float* __restrict__ lo, int* __restrict__ zero) {
+  if (zero && blockIdx.x == 0 && threadIdx.x == 0) *zero = 0;
   const int64_t e = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
   if (e >= count) return;
   const float v = B[e];
@@ -320,9 +321,9 @@ bool corr_tc_supported(const float* A, int p, int n, int64_t ldc) {
 }
 
 
-cudaError_t split_tf32(const float* B, int64_t count, float* hi, float* lo, cudaStream_t st) {
+cudaError_t split_tf32(const float* B, int64_t count, float* hi, float* lo, cudaStream_t st, int* zero) {
   if (count <= 0) return cudaSuccess;
-  split_kernel<<<(unsigned)((count + 255) / 256), 256, 0, st>>>(B, count, hi, lo);
+  split_kernel<<<(unsigned)((count + 255) / 256), 256, 0, st>>>(B, count, hi, lo, zero);
   return cudaGetLastError();
 }
 

@@ -62,7 +62,8 @@ struct SimtProblem {
 // C = A B^T of two problems with the same B: row tiles [0, tiles0) are P0's.
 __global__ void __launch_bounds__(NTHR, 2) gemm_nt_kernel(const SimtProblem P0, const SimtProblem P1,
                                                           int64_t tiles0, const float* __restrict__ B,
-                                                          int rows_b, int p) {
+                                                          int rows_b, int p, int* __restrict__ zero) {
+  if (zero && blockIdx.x == 0 && blockIdx.y == 0 && threadIdx.x == 0) *zero = 0;
   extern __shared__ __align__(16) float sm[];
   const bool second = (int64_t)blockIdx.x >= tiles0;
   const SimtProblem P = second ? P1 : P0;
@@ -135,7 +136,7 @@ __global__ void __launch_bounds__(NTHR, 2) gemm_nt_kernel(const SimtProblem P0, 
 
 cudaError_t gemm_nt_simt_pair(const float* A0, int64_t rows0, float* C0, int64_t ldc0, const float* A1,
                               int64_t rows1, float* C1, int64_t ldc1, const float* B, int rows_b, int p,
-                              cudaStream_t st) {
+                              cudaStream_t st, int* zero) {
   if (rows0 < 0) rows0 = 0;
   if (rows1 < 0 || !A1) rows1 = 0;
   const int64_t t0 = (rows0 + TM - 1) / TM, t1 = (rows1 + TM - 1) / TM;
@@ -145,7 +146,8 @@ cudaError_t gemm_nt_simt_pair(const float* A0, int64_t rows0, float* C0, int64_t
   if (e != cudaSuccess) return e;
   const dim3 grid((unsigned)(t0 + t1), (unsigned)((rows_b + TN - 1) / TN));
   gemm_nt_kernel<<<grid, NTHR, kSimtSmem, st>>>(SimtProblem{A0, rows0, C0, ldc0},
-                                                SimtProblem{A1, rows1, C1, ldc1}, t0, B, rows_b, p);
+                                                SimtProblem{A1, rows1, C1, ldc1}, t0, B, rows_b, p,
+                                                zero);
   return cudaGetLastError();
 }
 
@@ -168,7 +170,9 @@ namespace {
 constexpr int GT = 32, GK = 64;
 
 __global__ void __launch_bounds__(256) gram_kernel(const float* __restrict__ D, int n, int p,
-                                                   float* __restrict__ G, int tiles) {
+                                                   float* __restrict__ G, int tiles,
+                                                   int* __restrict__ zero) {
+  if (zero && blockIdx.x == 0 && threadIdx.x == 0) *zero = 0;
   __shared__ float Dj[GT][GK + 1];
   __shared__ float Dk[GT][GK + 1];
   // block b -> (jt, kt) with jt <= kt, row by row of the upper triangle
@@ -213,10 +217,10 @@ __global__ void __launch_bounds__(256) gram_kernel(const float* __restrict__ D, 
 
 }  // namespace
 
-cudaError_t gram_simt(const float* D, int n, int p, float* G, cudaStream_t st) {
+cudaError_t gram_simt(const float* D, int n, int p, float* G, cudaStream_t st, int* zero) {
   if (n <= 0) return cudaSuccess;
   const int tiles = (n + GT - 1) / GT;
-  gram_kernel<<<tiles * (tiles + 1) / 2, 256, 0, st>>>(D, n, p, G, tiles);
+  gram_kernel<<<tiles * (tiles + 1) / 2, 256, 0, st>>>(D, n, p, G, tiles, zero);
   return cudaGetLastError();
 }
 
