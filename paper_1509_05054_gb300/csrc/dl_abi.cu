@@ -401,6 +401,30 @@ cudaError_t enq_omp_res(dl_ctx* c, const float* Y, int64_t m, const float* D, in
   return e;
 }
 
+// Batch-OMP of m signals from their correlations A (BF16 rows when bf16) into the
+// slots from signal `off` on, by the kernel that is fastest for the shape
+// (cfg_omp_tm = 0: one warp per signal throughout).
+cudaError_t enq_batch_omp(dl_ctx* c, const float* A, bool bf16, const float* Y, int64_t m, int s,
+                          int64_t off, float* ores, float gap_tol) {
+  int32_t* idx = c->sidx + off * s;
+  float* val = c->sval + off * s;
+  int32_t* cnt = c->scnt + off;
+  const int cap = (int)c->m_max;
+  c->last_omp = 1;
+  if (c->cfg_omp_tm && dlk::omp_roll_supported(c->n, s))
+    return dlk::omp_roll(A, c->lda, c->G, c->n, Y, c->p, m, s, idx, val, cnt, ores, c->err, c->rs_list,
+                         c->rs_count, cap, gap_tol, c->st);
+  if (c->cfg_omp_tm && !has_prop(c) && dlk::omp_tm_supported(c->n, s))
+    return dlk::omp_batch_tm(c->cfg_omp_tm, A, bf16, c->lda, c->G, c->n, Y, c->p, m, s, idx, val, cnt,
+                             c->err, c->rs_list, c->rs_count, cap, c->st);
+  c->last_omp = 0;
+  if (c->cfg_omp_tm && dlk::omp_sub_supported(c->n, s, m))
+    return dlk::omp_sub(A, c->lda, c->G, c->n, Y, c->p, m, s, idx, val, cnt, ores, c->err, c->rs_list,
+                        c->rs_count, cap, c->st);
+  return dlk::omp_batch(A, c->lda, c->G, c->n, Y, c->p, m, s, idx, val, cnt, c->err, c->rs_list,
+                        c->rs_count, cap, c->cfg_omp_warps, ores, gap_tol, c->st);
+}
+
 cudaError_t enq_omp(dl_ctx* c, const float* Y, int64_t m, const float* D, int s) {
   if (use_res(c, Y, D, s, m)) return enq_omp_res(c, Y, m, D, s);
   const bool tc = tc_ok(c, Y, D);
@@ -433,20 +457,8 @@ cudaError_t enq_omp(dl_ctx* c, const float* Y, int64_t m, const float* D, int s)
     c->omp_kernels[0] = (tc ? 2 : 1) + (lp_ok(c) ? 2 : 1) + 2;
   }
   mark(c, 2);
-  const bool tm = c->cfg_omp_tm && !has_prop(c) && dlk::omp_tm_supported(c->n, s);
-  const bool roll = c->cfg_omp_tm && dlk::omp_roll_supported(c->n, s);
-  c->last_omp = tm || roll ? 1 : 0;
-  if (roll)
-    e = dlk::omp_roll(c->A0, c->lda, c->G, c->n, Y, c->p, m, s, c->sidx, c->sval, c->scnt,
-                      has_prop(c) ? c->rr_ref : nullptr, c->err, c->rs_list, c->rs_count,
-                      (int)c->m_max, lp_ok(c) ? 0.f : dlk::kGapTol, c->st);
-  else if (tm)
-    e = dlk::omp_batch_tm(c->cfg_omp_tm, c->A0, c->a0_bf16, c->lda, c->G, c->n, Y, c->p, m, s, c->sidx, c->sval,
-                          c->scnt, c->err, c->rs_list, c->rs_count, (int)c->m_max, c->st);
-  else
-    e = dlk::omp_batch(c->A0, c->lda, c->G, c->n, Y, c->p, m, s, c->sidx, c->sval, c->scnt, c->err,
-                       c->rs_list, c->rs_count, (int)c->m_max, c->cfg_omp_warps,
-                       has_prop(c) ? c->rr_ref : nullptr, lp_ok(c) ? 0.f : dlk::kGapTol, c->st);
+  e = enq_batch_omp(c, c->A0, c->a0_bf16, Y, m, s, 0, has_prop(c) ? c->rr_ref : nullptr,
+                    lp_ok(c) ? 0.f : dlk::kGapTol);
   if (e != cudaSuccess) return e;
   e = dlk::omp_resolve64(Y, c->p, D, c->G, lp_ok(c) ? nullptr : c->A0, c->lda, c->n, s,
                          c->rs_list, c->rs_count, (int)c->m_max, c->sidx, c->sval, c->scnt, c->st);
@@ -638,7 +650,6 @@ cudaError_t enq_omp_staged(dl_ctx* c, const float* hostY, const float* dY, int64
     if ((e = cudaEventRecord(c->ev_chunk[q], c->st2)) != cudaSuccess) return e;
   }
   mark(c, 2);
-  const bool roll = c->cfg_omp_tm && dlk::omp_roll_supported(c->n, s);
   bool first = true;
   for (int q = 0; q < dl_ctx::kChunks; ++q) {
     const int64_t off = offs[q], mk = offs[q + 1] - offs[q];
@@ -652,18 +663,7 @@ cudaError_t enq_omp_staged(dl_ctx* c, const float* hostY, const float* dY, int64
     if (e != cudaSuccess) return e;
     first = false;
     if ((e = cudaMemsetAsync(c->rs_count, 0, sizeof(int), c->st)) != cudaSuccess) return e;
-    if (roll)
-      e = dlk::omp_roll(Aq, c->lda, c->G, c->n, Yq, c->p, mk, s, c->sidx + off * s,
-                        c->sval + off * s, c->scnt + off, nullptr, c->err, c->rs_list, c->rs_count,
-                        (int)c->m_max, dlk::kGapTol, c->st);
-    else if (c->cfg_omp_tm && dlk::omp_tm_supported(c->n, s))
-      e = dlk::omp_batch_tm(c->cfg_omp_tm, Aq, false, c->lda, c->G, c->n, Yq, c->p, mk, s, c->sidx + off * s,
-                            c->sval + off * s, c->scnt + off, c->err, c->rs_list, c->rs_count,
-                            (int)c->m_max, c->st);
-    else
-      e = dlk::omp_batch(Aq, c->lda, c->G, c->n, Yq, c->p, mk, s, c->sidx + off * s,
-                         c->sval + off * s, c->scnt + off, c->err, c->rs_list, c->rs_count,
-                         (int)c->m_max, c->cfg_omp_warps, nullptr, dlk::kGapTol, c->st);
+    e = enq_batch_omp(c, Aq, false, Yq, mk, s, off, nullptr, dlk::kGapTol);
     if (e != cudaSuccess) return e;
     e = dlk::omp_resolve64(Yq, c->p, D, c->G, Aq, c->lda, c->n, s, c->rs_list, c->rs_count,
                            (int)c->m_max, c->sidx + off * s, c->sval + off * s, c->scnt + off,
@@ -672,7 +672,6 @@ cudaError_t enq_omp_staged(dl_ctx* c, const float* hostY, const float* dY, int64
     k += 3;
   }
   mark(c, 3);
-  c->last_omp = c->cfg_omp_tm && (roll || dlk::omp_tm_supported(c->n, s)) ? 1 : 0;
   *kernels = k;
   return cudaSuccess;
 }

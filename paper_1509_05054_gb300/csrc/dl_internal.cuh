@@ -106,6 +106,12 @@ cudaError_t omp_batch_tm(int q, const void* A0, bool a0_bf16, int64_t lda, const
                          int32_t* cnt, int* err, int* rs_list, int* rs_count, int rs_cap,
                          cudaStream_t st);
 
+// The arithmetic of omp_batch with several signals per warp (k_omp_sub.cu); supported
+// means that it is also the faster one.
+bool omp_sub_supported(int n, int s, int64_t m);
+cudaError_t omp_sub(const float* A0, int64_t lda, const float* G, int n, const float* Y, int p, int64_t m,
+                    int s, int32_t* idx, float* val, int32_t* cnt, float* ores, int* err, int* rs_list,
+                    int* rs_count, int rs_cap, cudaStream_t st);
 // The arithmetic of omp_batch with rolled loops and the vectors in TMEM and shared
 // memory (k_omp_roll.cu); supported means that it is also the faster one.
 bool omp_roll_supported(int n, int s);
