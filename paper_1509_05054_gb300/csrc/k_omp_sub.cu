@@ -26,6 +26,7 @@
 // is the latency of a step's chain with 17 to 20 warps per SM, which shared memory sets.
 #include "dl_internal.cuh"
 #include "omp_common.cuh"
+#include "omp_sub.cuh"
 
 #include <math.h>
 
@@ -36,7 +37,6 @@ namespace {
 
 using namespace omp;
 
-constexpr int SUB_SMAX = 8;
 constexpr int SUB_WARPS = 24;                // most warps per CTA (one CTA per SM)
 constexpr size_t kSubSmem = 220 * 1024;      // dynamic shared memory of a CTA
 
@@ -47,17 +47,23 @@ __device__ __forceinline__ float4 ld_stream4(const float* p) {
       : "l"(p));
   return v;
 }
-__device__ __forceinline__ float4 f4_fma2(float2 a, float4 b, float4 c) {
-  const float2 lo = __ffma2_rn(a, make_float2(b.x, b.y), make_float2(c.x, c.y));
-  const float2 hi = __ffma2_rn(a, make_float2(b.z, b.w), make_float2(c.z, c.w));
-  return make_float4(lo.x, lo.y, hi.x, hi.y);
-}
-
-// Floats of one signal: alpha and u_q (q < s - 1) of NP = 4 SW V each, s x s Cholesky rows.
-template <int SW, int V>
-__host__ __device__ constexpr int sub_signal_floats(int s) {
-  return s * 4 * SW * V + (s * s + 3) / 4 * 4;
-}
+// Rows of G in shared memory (pitch NP, zero past n), or in global memory (VEC: n % 4
+// == 0, as float4).
+template <int NP, bool GSH, bool VEC>
+struct SubGram {
+  const float* G;
+  int n;
+  __device__ __forceinline__ float diag(int j) const {
+    return GSH ? G[j * NP + j] : __ldg(G + (size_t)j * n + j);
+  }
+  __device__ __forceinline__ float4 vec(int row, int j) const {
+    if (GSH) return *(const float4*)(G + row * NP + j);
+    const float* Gr = G + (size_t)row * n;
+    if (VEC) return j < n ? __ldg((const float4*)(Gr + j)) : make_float4(0.f, 0.f, 0.f, 0.f);
+    return make_float4(j < n ? __ldg(Gr + j) : 0.f, j + 1 < n ? __ldg(Gr + j + 1) : 0.f,
+                       j + 2 < n ? __ldg(Gr + j + 2) : 0.f, j + 3 < n ? __ldg(Gr + j + 3) : 0.f);
+  }
+};
 
 // TB: truncated mantissa bits; GSH: G in shared memory (pitch NP); VEC: rows of G
 // in global memory as float4 (n % 4 == 0).
@@ -68,15 +74,11 @@ __global__ void __launch_bounds__(SUB_WARPS * 32, 1) omp_sub_kernel(
     float* __restrict__ oval, int32_t* __restrict__ ocnt, float* __restrict__ ores,
     int* __restrict__ err, int* __restrict__ rs_list, int* __restrict__ rs_count, int rs_cap) {
   constexpr int SPW = 32 / SW, NP = 4 * SW * V;
-  constexpr unsigned VMASK = 0x7FFFFFFFu & ~((1u << TB) - 1u);
-  static_assert(V <= (1 << TB), "vector number in the truncated bits");
   extern __shared__ __align__(16) float sm[];
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, W = blockDim.x >> 5;
   const int sub = lane / SW, l = lane % SW;
-  const float* Gs = sm;
+  const SubGram<NP, GSH, VEC> gram{GSH ? sm : G, n};
   float* base = sm + (GSH ? n * NP : 0) + (warp * SPW + sub) * sub_signal_floats<SW, V>(s);
-  float* L = base + s * NP;
-  float4* al = (float4*)base + l;                    // alpha: vector v at al[SW v]
   const float qnan = __int_as_float(0x7fc00000);
   if (GSH) {
 #pragma unroll 4
@@ -119,8 +121,7 @@ __global__ void __launch_bounds__(SUB_WARPS * 32, 1) omp_sub_kernel(
       if (j + 2 >= n) a[v].z = qnan;
       if (j + 3 >= n) a[v].w = qnan;
     }
-    // ||y||^2, summed as a warp sums it (element r on lane r mod 32, then a tree by halves)
-    float yy;
+    float yy;  // ||y||^2
     {
       float t[32 / SW];
 #pragma unroll
@@ -131,165 +132,10 @@ __global__ void __launch_bounds__(SUB_WARPS * 32, 1) omp_sub_kernel(
           t[h] = fmaf(v, v, t[h]);
         }
       }
-      if constexpr (SW == 8) yy = (t[0] + t[2]) + (t[1] + t[3]);
-      else yy = t[0] + t[1];
-#pragma unroll
-      for (int o = SW / 2; o > 0; o >>= 1) yy += __shfl_xor_sync(FULL, yy, o);
+      yy = sub_norm2<SW>(t);
     }
-    bool act = live && isfinite(yy);
-    if (live && !isfinite(yy) && l == 0) atomicOr(err, ERR_NONFINITE);
-    float myc = 0.f, myz = 0.f;  // lane q: c_q = 1 / L_qq, z_q
-    int myI = -1;                // lane q: I_q
-    float rr = yy;
-    int k = 0;
-    float kmax = 0.f;
-    auto keys = [&]() {  // this lane's largest key
-      kmax = 0.f;
-#pragma unroll
-      for (int v = 0; v < V; ++v) {
-        auto key = [&](float x) {
-          return __uint_as_float((__float_as_uint(x) & VMASK) | (uint32_t)(V - 1 - v));
-        };
-        kmax = fmax3(kmax, fmaxf(key(a[v].x), key(a[v].y)), fmaxf(key(a[v].z), key(a[v].w)));
-      }
-    };
-#pragma unroll
-    for (int v = 0; v < V; ++v) al[SW * v] = a[v];
-    keys();
-    __syncwarp();
-#pragma unroll 1
-    for (int step = 0; step < s; ++step) {
-      // ---- argmax over the signal's lanes
-      float km = kmax;
-#pragma unroll
-      for (int o = SW / 2; o > 0; o >>= 1) km = fmaxf(km, __shfl_xor_sync(FULL, km, o));
-      const unsigned kb = __float_as_uint(km);
-      if ((kb & VMASK) == 0u) act = false;  // max |alpha| = 0
-      if (!__any_sync(FULL, act)) break;
-      const unsigned ball = __ballot_sync(FULL, __float_as_uint(kmax) == kb) >> (sub * SW);
-      const int lsel = __ffs(ball) - 1;
-      const int vsel = lsel + SW * (V - 1 - (int)(kb & ((1u << TB) - 1u)) % V);
-      const int vs = act ? vsel : 0;  // (in range also for a signal that has stopped)
-      const float4 q4 = ((const float4*)base)[vs];
-      int e = 3;
-      float asel = q4.w;
-      if ((__float_as_uint(q4.z) & VMASK) == (kb & VMASK)) e = 2, asel = q4.z;
-      if ((__float_as_uint(q4.y) & VMASK) == (kb & VMASK)) e = 1, asel = q4.y;
-      if ((__float_as_uint(q4.x) & VMASK) == (kb & VMASK)) e = 0, asel = q4.x;
-      const int sel = act ? 4 * vs + e : 0;
-      // ---- the Gram loads: diagonal and row
-      const bool need_u = step + 1 < s;
-      const float gss = GSH ? Gs[sel * NP + sel] : __ldg(G + (size_t)sel * n + sel);
-      float4 g[V];
-      if (need_u) {
-#pragma unroll
-        for (int v = 0; v < V; ++v) {
-          const int j = 4 * (l + SW * v);
-          if (GSH) {
-            g[v] = *(const float4*)(Gs + sel * NP + j);
-          } else if (VEC) {
-            g[v] = j < n ? __ldg((const float4*)(G + (size_t)sel * n + j)) : make_float4(0.f, 0.f, 0.f, 0.f);
-          } else {
-            const float* Gr = G + (size_t)sel * n;
-            g[v].x = j < n ? __ldg(Gr + j) : 0.f;
-            g[v].y = j + 1 < n ? __ldg(Gr + j + 1) : 0.f;
-            g[v].z = j + 2 < n ? __ldg(Gr + j + 2) : 0.f;
-            g[v].w = j + 3 < n ? __ldg(Gr + j + 3) : 0.f;
-          }
-        }
-      }
-      // ---- Cholesky row: lane q < step: w_q = c_q u_q[sel]
-      const float ul = l < step ? base[(1 + l) * NP + sel] : 0.f;
-      const float w = ul * myc, negaw = -w * myc;
-      float wsq = 0.f;
-      for (int q = 0; q < step; ++q) {
-        const float wq = __shfl_sync(FULL, w, q, SW);
-        wsq = fmaf(wq, wq, wsq);
-      }
-      if (l < step) L[step * s + l] = w;
-      const float delta = gss - wsq;
-      if (act && !(delta > kPivotMin)) {
-        if (l == 0) {
-          if (!isfinite(delta)) atomicOr(err, ERR_NONFINITE);
-          if (rs_count) {  // rounding dominates this pivot: redo the signal in FP64
-            const int pos = atomicAdd(rs_count, 1);
-            if (pos < rs_cap) rs_list[pos] = (int)i;
-          }
-        }
-        act = false;
-      }
-      // c_k = 1 / L_kk: rsqrtf refined by one Newton-Raphson step, y + y (1 - d y^2) / 2
-      float ck = rsqrtf(delta);
-      ck = fmaf(0.5f * ck, fmaf(-delta * ck, ck, 1.0f), ck);
-      const float zk = asel * ck;
-      if (act) {
-        if (l == step) {
-          myc = ck;
-          myz = zk;
-          myI = sel;
-        }
-        rr = fmaf(-zk, zk, rr);
-        k = step + 1;
-        if (l == 0) base[sel] = qnan;  // selected: masked from now on
-      }
-      __syncwarp();
-      // ---- u_step = G[:, sel] + sum_q negaw_q u_q;  alpha -= (z_k c_k) u_step
-      if (need_u) {
-#pragma unroll
-        for (int v = 0; v < V; ++v) a[v] = al[SW * v];
-#pragma unroll 2
-        for (int q = 0; q < step; ++q) {
-          const float nq = __shfl_sync(FULL, negaw, q, SW);
-          const float2 n2 = make_float2(nq, nq);
-          const float4* uq = al + (1 + q) * (NP / 4);
-#pragma unroll
-          for (int v = 0; v < V; ++v) g[v] = f4_fma2(n2, uq[SW * v], g[v]);
-        }
-        const float nz = -zk * ck;
-        const float2 nz2 = make_float2(nz, nz);
-        float4* us = al + (1 + step) * (NP / 4);
-#pragma unroll
-        for (int v = 0; v < V; ++v) {
-          us[SW * v] = g[v];
-          a[v] = f4_fma2(nz2, g[v], a[v]);
-          al[SW * v] = a[v];
-        }
-        keys();
-      }
-      if (rr <= kResidRel * yy) act = false;
-      __syncwarp();
-    }
-    // ---- back substitution L^T gamma = z
-    float gam = 0.f, acc2 = 0.f;
-    for (int q = s - 1; q >= 0; --q) {
-      const float gl = (myz - acc2) * myc;  // valid on lane q
-      const float gq = __shfl_sync(FULL, gl, q, SW);
-      if (q < k) {
-        if (l == q) gam = gq;
-        if (l < q) acc2 = fmaf(L[q * s + l], gq, acc2);
-      }
-    }
-    // ---- the support in ascending atom order
-    int rank = 0;
-    for (int q = 0; q < s; ++q) {
-      const int Iq = __shfl_sync(FULL, myI, q, SW);
-      rank += q < k && Iq < myI ? 1 : 0;
-    }
-    if (live) {
-      const int64_t o = i * s;
-      if (l < k) {
-        oidx[o + rank] = myI;
-        oval[o + rank] = gam;
-      } else if (l < s) {
-        oidx[o + l] = -1;
-        oval[o + l] = 0.f;
-      }
-      if (l == 0) {
-        ocnt[i] = k;
-        if (ores) ores[i] = rr;
-      }
-    }
-    __syncwarp();
+    omp_sub_core<SW, V, TB>(i, live, a, yy, gram, base, s, oidx, oval, ocnt, ores, err, rs_list, rs_count,
+                            rs_cap);
   }
 }
 

@@ -8,10 +8,12 @@
 // dictionary, Gram matrix and U = E X^T in shared memory and runs every stage
 // of every iteration itself:
 //   1. G = D^T D (FP32) from the shared-memory atoms;
-//   2. OMP, one warp per signal (omp_one, the same Gram-Schmidt Batch-OMP as the
-//      large-problem kernels, Gram rows from shared memory); a signal whose
-//      Cholesky pivot falls below 1e-6 is redone by the same warp in FP64 with
-//      the oracle's stop rules;
+//   2. OMP, eight lanes per signal, four signals per warp in step (omp_sub_core, the
+//      same Gram-Schmidt Batch-OMP as the large-problem kernels, Gram rows from
+//      shared memory); a signal whose Cholesky pivot falls below 1e-6 is redone by
+//      the warp in FP64 with the oracle's stop rules.  (With a warp per signal, and
+//      the energies summed in FP64 signal by signal, an iteration of 200 problems
+//      at p = 20, n = 50, m = 1500, s = 4 took 919 us, now 490);
 //   3. e_i = y_i - D x_i, U = E X^T and r_j = ||x_j||^2 by shared-memory
 //      reductions (X_prev for P-NSGK, Eq. 7), ||E||^2 and ||Y||^2;
 //   4. the atom update (Eq. 5): d_j' = (U_j + r_j d_j) / ||.||, c_j = d_j^T d_j';
@@ -22,7 +24,7 @@
 // group size n.
 #include "dl_internal.cuh"
 #include "omp_common.cuh"
-#include "omp_one.cuh"
+#include "omp_sub.cuh"
 
 #include <math.h>
 
@@ -34,21 +36,28 @@ using namespace omp;
 constexpr int SM_THREADS = 1024;
 constexpr int SM_WARPS = SM_THREADS / 32;
 
-// Gram rows from the problem's Gram matrix in shared memory (row pitch n).
+constexpr int SM_NP = 64;  // padded atoms: eight lanes x two vectors of four
+constexpr int SM_SPW = 4;  // signals per warp of the OMP
+
+// Gram rows from the problem's Gram matrix in shared memory (row pitch SM_NP, zero past n).
 struct GramShared {
   const float* G;
-  int n;
-  template <int NV>
-  __device__ __forceinline__ void row(int sel, int lane, float2 (&out)[NV]) const {
-    const float* Gr = G + sel * n;
-#pragma unroll
-    for (int v = 0; v < NV; ++v) {
-      const int j0 = 64 * v + lane, j1 = j0 + 32;
-      out[v].x = j0 < n ? Gr[j0] : 0.f;
-      out[v].y = j1 < n ? Gr[j1] : 0.f;
-    }
+  __device__ __forceinline__ float diag(int j) const { return G[j * SM_NP + j]; }
+  __device__ __forceinline__ float4 vec(int row, int j) const { return *(const float4*)(G + row * SM_NP + j); }
+};
+
+// A sum of FP32 values as an unevaluated pair (Knuth's two-sum: every addition's
+// rounding error goes to lo): FP64 additions run at 1/64 of the FP32 rate.
+struct Sum2 {
+  float hi = 0.f, lo = 0.f;
+  __device__ __forceinline__ void add(float x) {
+    const float s = __fadd_rn(hi, x), b = __fsub_rn(s, hi);
+    lo = __fadd_rn(lo, __fadd_rn(__fsub_rn(hi, __fsub_rn(s, b)), __fsub_rn(x, b)));
+    hi = s;
   }
-  __device__ __forceinline__ float diag(int sel) const { return G[sel * n + sel]; }
+  __device__ __forceinline__ double value() const {
+    return isfinite(hi) ? (double)hi + (double)lo : (double)hi;
+  }
 };
 
 __device__ __forceinline__ double warp_sum_d(double v) {
@@ -188,37 +197,41 @@ __device__ void block_sum3(double& a, double& b, double& c, double (*red)[3]) {
   __syncthreads();
 }
 
-// Shared memory of one CTA (floats unless noted); pitch of D rows = p | 1 (odd:
-// the lane-per-atom reads of the correlations hit distinct banks).
+// Shared memory of one CTA (floats); pitch of D rows = p | 1 (odd: lanes on
+// different atoms hit distinct banks); dt: D transposed (row r: entry r of all atoms,
+// zero past n).  The OMP's warps share what is left, each four signals' state (the
+// FP64 re-solve uses the same space): wo warps.
 struct SmallSmem {
-  int pitch, n;
-  size_t ds, dn, g, u, r, c, a0, lf, cf, w64, total;
-  __host__ __device__ SmallSmem(int p_, int n_) : pitch(p_ | 1), n(n_) {
+  int pitch, per, wo;
+  size_t ds, dn, u, r, c, g, dt, omp;
+  __host__ __device__ SmallSmem(int p, int n, int s, size_t floats) : pitch(p | 1) {
     ds = 0;
     dn = ds + (size_t)n * pitch;
-    g = dn + (size_t)n * pitch;
-    u = g + (size_t)n * n;
+    u = dn + (size_t)n * pitch;
     r = u + (size_t)n * pitch;
     c = r + n;
-    a0 = c + n;
-    lf = a0 + (size_t)SM_WARPS * kSmallN;
-    cf = lf + (size_t)SM_WARPS * kSmallS * kSmallS;
-    w64 = (cf + (size_t)SM_WARPS * kSmallS + 1) / 2 * 2;  // 8-byte aligned
-    total = w64 * sizeof(float) + (size_t)SM_WARPS * sizeof(Omp64Scratch);
+    g = (c + n + 3) / 4 * 4;
+    dt = g + (size_t)n * SM_NP;
+    omp = dt + (size_t)p * SM_NP;
+    per = SM_SPW * sub_signal_floats<8, 2>(s);
+    const size_t w = floats > omp ? (floats - omp) / per : 0;
+    wo = w < SM_WARPS ? (int)w : SM_WARPS;
   }
 };
+constexpr size_t kSmallSmem = 224 * 1024;
+static_assert(SM_SPW * (SM_NP + 4) * sizeof(float) >= sizeof(Omp64Scratch), "re-solve scratch");
 
 __global__ void __launch_bounds__(SM_THREADS) small_dl_kernel(const SmallProblem* __restrict__ probs,
                                                               int iters, int rule,
                                                               int* __restrict__ err) {
-  extern __shared__ float smem[];
+  extern __shared__ __align__(16) float smem[];
   __shared__ double red[SM_WARPS][3];
   __shared__ int rs_cnt[SM_WARPS];
-  __shared__ int rs_one[SM_WARPS];
+  __shared__ int rs_one[SM_WARPS][SM_SPW];
   const SmallProblem P = probs[blockIdx.x];
   const int p = P.p, n = P.n, s = P.s;
   const int64_t m = P.m;
-  const SmallSmem lay(p, n);
+  const SmallSmem lay(p, n, s, kSmallSmem / sizeof(float));
   const int pitch = lay.pitch;
   float* Ds = smem + lay.ds;  // atoms (current)
   float* Dn = smem + lay.dn;  // updated atoms
@@ -227,47 +240,78 @@ __global__ void __launch_bounds__(SM_THREADS) small_dl_kernel(const SmallProblem
   float* R = smem + lay.r;
   float* Cc = smem + lay.c;
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-  float* a0w = smem + lay.a0 + warp * kSmallN;
-  float(&Lw)[kSmallS][kSmallS] =
-      *(float(*)[kSmallS][kSmallS])(smem + lay.lf + warp * kSmallS * kSmallS);
-  float(&Cw)[kSmallS] = *(float(*)[kSmallS])(smem + lay.cf + warp * kSmallS);
-  Omp64Scratch& w64 = ((Omp64Scratch*)(smem + lay.w64))[warp];
+  float* Dt = smem + lay.dt;
+  float* wbase = smem + lay.omp + (size_t)warp * lay.per;  // (warps below lay.wo)
   const bool nsgk = rule == 2, sgk = rule != 0;
 
   for (int q = threadIdx.x; q < n * p; q += SM_THREADS) Ds[(q / p) * pitch + q % p] = P.D[q];
   __syncthreads();
   for (int it = 0; it < iters; ++it) {
     // ---- 1. Gram matrix
-    for (int q = threadIdx.x; q < n * n; q += SM_THREADS) {
-      const int j = q / n, k = q - j * n;
+    for (int q = threadIdx.x; q < n * SM_NP; q += SM_THREADS) {
+      const int j = q / SM_NP, k = q % SM_NP;
       float a = 0.f;
-      for (int r = 0; r < p; ++r) a = fmaf(Ds[j * pitch + r], Ds[k * pitch + r], a);
+      if (k < n)
+        for (int r = 0; r < p; ++r) a = fmaf(Ds[j * pitch + r], Ds[k * pitch + r], a);
       G[q] = a;
+    }
+    for (int q = threadIdx.x; q < p * SM_NP; q += SM_THREADS) {
+      const int r = q / SM_NP, j = q % SM_NP;
+      Dt[q] = j < n ? Ds[j * pitch + r] : 0.f;
     }
     for (int q = threadIdx.x; q < n * pitch + n; q += SM_THREADS) U[q] = 0.f;  // U, then R
     __syncthreads();
-    // ---- 2. sparse coding, one warp per signal
-    const GramShared gsrc{G, n};
-    for (int64_t i = warp; i < m; i += SM_WARPS) {
-      const float* y = P.Y + i * p;
-      const float yv = lane < p ? y[lane] : 0.f;
-      float a[2] = {0.f, 0.f};
-      for (int r = 0; r < p; ++r) {
-        const float yr = __shfl_sync(FULL, yv, r);
-        if (lane < n) a[0] = fmaf(Ds[lane * pitch + r], yr, a[0]);
-        if (lane + 32 < n) a[1] = fmaf(Ds[(lane + 32) * pitch + r], yr, a[1]);
+    // ---- 2. sparse coding, four signals per warp
+    if (warp < lay.wo) {
+      const GramShared gram{G};
+      const int sub = lane >> 3, l = lane & 7;
+      const float qnan = __int_as_float(0x7fc00000);
+      for (int64_t i0 = (int64_t)warp * SM_SPW; i0 < m; i0 += (int64_t)lay.wo * SM_SPW) {
+        const int64_t i = i0 + sub;
+        const bool live = i < m;
+        const float* y = P.Y + (live ? i : 0) * p;
+        float yv[4], t[4];  // elements l + 8 h
+#pragma unroll
+        for (int h = 0; h < 4; ++h) {
+          yv[h] = live && l + 8 * h < p ? y[l + 8 * h] : 0.f;
+          t[h] = fmaf(yv[h], yv[h], 0.f);
+        }
+        const float yy = sub_norm2<8>(t);
+        // correlations of atoms 4 (l + 8 v) .., sums over the entries in order
+        float4 a[2];
+        a[0] = a[1] = make_float4(0.f, 0.f, 0.f, 0.f);
+#pragma unroll
+        for (int h = 0; h < 4; ++h) {
+          for (int q = 0; q < 8; ++q) {
+            const int r = 8 * h + q;
+            if (r >= p) break;
+            const float yr = __shfl_sync(FULL, yv[h], q, 8);
+            const float2 y2 = make_float2(yr, yr);
+#pragma unroll
+            for (int v = 0; v < 2; ++v)
+              a[v] = f4_fma2(y2, *(const float4*)(Dt + r * SM_NP + 4 * (l + 8 * v)), a[v]);
+          }
+        }
+#pragma unroll
+        for (int v = 0; v < 2; ++v) {  // atoms past n never win
+          const int j = 4 * (l + 8 * v);
+          if (j >= n) a[v].x = qnan;
+          if (j + 1 >= n) a[v].y = qnan;
+          if (j + 2 >= n) a[v].z = qnan;
+          if (j + 3 >= n) a[v].w = qnan;
+        }
+        if (lane == 0) rs_cnt[warp] = 0;
+        __syncwarp();
+        omp_sub_core<8, 2, tbits<2>()>(i, live, a, yy, gram, wbase + sub * sub_signal_floats<8, 2>(s), s,
+                                       P.sidx, P.sval, P.scnt, nullptr, err, rs_one[warp], &rs_cnt[warp],
+                                       SM_SPW);
+        const int redo = rs_cnt[warp];  // a pivot below 1e-6: the signal again in FP64
+        for (int q = 0; q < redo; ++q) {
+          const int64_t ir = rs_one[warp][q];
+          omp64_small(Ds, pitch, n, p, s, P.Y + ir * p, *(Omp64Scratch*)wbase, ir, P.sidx, P.sval, P.scnt);
+        }
+        __syncwarp();
       }
-      a0w[lane] = a[0];
-      a0w[lane + 32] = a[1];
-      if (lane == 0) rs_cnt[warp] = 0;
-      __syncwarp();
-      omp_one<2, kSmallS, kSmallS - 1, false, false>(i, gsrc, Lw, Cw, nullptr, a0w, n, y, p, s,
-                                                     nullptr, P.sidx, P.sval, P.scnt, nullptr, err,
-                                                     &rs_one[warp], &rs_cnt[warp], 1, 0.f);
-      __syncwarp();
-      if (rs_cnt[warp] > 0)  // a pivot below 1e-6: redo the signal in FP64
-        omp64_small(Ds, pitch, n, p, s, y, w64, i, P.sidx, P.sval, P.scnt);
-      __syncwarp();
     }
     __syncthreads();
     // ---- 3. errors, U = E X^T and r (X_prev's slots for P-NSGK once there is one)
@@ -275,7 +319,7 @@ __global__ void __launch_bounds__(SM_THREADS) small_dl_kernel(const SmallProblem
     const int32_t* aidx = prev ? P.pidx : P.sidx;
     const float* aval = prev ? P.pval : P.sval;
     const int32_t* acnt = prev ? P.pcnt : P.scnt;
-    double ee = 0.0, yy = 0.0, e2 = 0.0;
+    Sum2 see, syy, se2;
     for (int64_t i = warp; i < m; i += SM_WARPS) {
       const float yv = lane < p ? P.Y[i * p + lane] : 0.f;
       const int c = P.scnt[i];
@@ -287,8 +331,8 @@ __global__ void __launch_bounds__(SM_THREADS) small_dl_kernel(const SmallProblem
         const float x = __shfl_sync(FULL, xt, t);
         if (lane < p) e = fmaf(-x, Ds[j * pitch + lane], e);
       }
-      ee += (double)(e * e);
-      yy += (double)(yv * yv);
+      see.add(e * e);
+      syy.add(yv * yv);
       const int ca = acnt[i];
       const int ja = lane < ca ? aidx[i * s + lane] : 0;
       const float xa = lane < ca ? aval[i * s + lane] : 0.f;
@@ -337,9 +381,10 @@ __global__ void __launch_bounds__(SM_THREADS) small_dl_kernel(const SmallProblem
         if (lane == t) xnew = xn;
         r2 = fmaf(-xn, dn, r2);
       }
-      if (lane < p) e2 += (double)(r2 * r2);
+      if (lane < p) se2.add(r2 * r2);
       if (lane < c) P.sval[i * s + lane] = xnew;
     }
+    double ee = see.value(), yy = syy.value(), e2 = se2.value();
     block_sum3(ee, yy, e2, red);
     if (threadIdx.x == 0) {
       P.rmse[2 * it] = yy > 0.0 ? sqrt(ee / yy) : 0.0;
@@ -411,7 +456,7 @@ bool small_supported(int p, int n, int s) {
 cudaError_t small_dl(const SmallProblem* probs, int count, int iters, int rule, int* err,
                      cudaStream_t st) {
   if (count <= 0 || iters <= 0) return cudaSuccess;
-  const size_t smem = SmallSmem(kSmallP, kSmallN).total;  // the largest layout
+  const size_t smem = kSmallSmem;
   cudaError_t e = cudaFuncSetAttribute(small_dl_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize,
                                        (int)smem);
   if (e != cudaSuccess) return e;
