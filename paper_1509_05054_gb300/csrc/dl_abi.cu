@@ -57,7 +57,7 @@ struct dl_ctx {
   int64_t lda = 0;  // row stride of the correlation matrix A0 (floats)
   // workspace
   float* G = nullptr;
-  float* A0 = nullptr;   // m_max x max(lda, p): alpha0, then the errors of the atom update
+  float* A0 = nullptr;   // m_max x max(lda, padded p): alpha0, then the errors of the atom update
   int jau_kernels = 5;   // kernel launches of the last enqueued JAU update
   int ntilde = 0;        // group size of the atom update (0 or n: all atoms at once)
   int rule = DL_RULE_AKSVD;  // atom update rule
@@ -177,7 +177,7 @@ void free_ctx(dl_ctx* c) {
   if (c->st2) cudaStreamDestroy(c->st2);
   void* ptrs[] = {c->G, c->A0, c->Dhi, c->Dlo, c->Ylp, c->Ysc, c->Dlp, c->Dsc, c->rs_list,
                   c->rs_count, c->sidx, c->sval, c->scnt, c->bsum, c->err, c->iter, c->rmse,
-                  c->jw.Upart, c->jw.U, c->jw.Ucopy, c->jw.epart_a, c->jw.epart_b, c->jw.Dn, c->jw.C,
+                  c->jw.Upart, c->jw.U, c->jw.Ucopy, c->jw.epart_a, c->jw.epart_b, c->jw.Dn, c->jw.Dp, c->jw.C,
                   c->hY, c->hD, c->hcolptr, c->hrowidx, c->hval, c->pidx, c->pval, c->pcnt,
                   c->pvalid, c->D0};
   for (void* q : ptrs)
@@ -477,7 +477,7 @@ cudaError_t enq_jau(dl_ctx* c, const float* Y, int64_t m, float* D, int s, const
   c->jw.det = c->deterministic && dlk::jau_det_supported(c->p, c->n, s, Y, D);
   // the errors go where the coding pass kept alpha0, which nothing reads any more
   const bool plain = group_size(c) == c->n && c->rule != DL_RULE_NSGK && !c->jw.det && m > 0;
-  c->jw.E = plain && dlk::jau_plain_supported(m, c->p, c->n, s, Y, D) ? c->A0 : nullptr;
+  c->jw.E = plain && dlk::jau_plain_supported(m, c->p, c->n, s) ? c->A0 : nullptr;
   c->jw.nb_accum = c->jw.det ? (int)dlk::jau_det_ranges(m, c->p, c->n, s)
                    : c->jw.E ? dlk::jau_plain_blocks(c->p)
                              : dlk::jau_accum_blocks(c->p, c->n, c->cfg_acc_mult);
@@ -496,7 +496,8 @@ cudaError_t enq_jau(dl_ctx* c, const float* Y, int64_t m, float* D, int s, const
                                     cudaMemcpyDeviceToDevice, c->st)) != cudaSuccess)
     return e0;
   // (groups need the float4 passes; the entry points check this before enqueuing)
-  c->jw.copies = !c->jw.det && dlk::jau_vec4(c->p, Y, D);
+  c->jw.copies = c->jw.E || (!c->jw.det && dlk::jau_vec4(c->p, Y, D));
+  c->jw.padded = c->jw.E && !dlk::jau_vec4(c->p, Y, D);
   c->jau_kernels = (dlk::jau_launches(c->jw) - 1) * ngroups + 1;
   mark(c, 4);
   cudaError_t e = cudaSuccess;
@@ -851,12 +852,13 @@ int dl_init(dl_ctx** out, int p, int n, int64_t m_max, int s_max, int precision,
   const size_t ulen = dlk::jau_ulen(p, n);
   size_t nslices = dlk::jau_accum_smem(p, n) > 0 ? (size_t)c->jw.nb_accum : 1;
   if (nslices < (size_t)nbd) nslices = (size_t)nbd;
-  bool ok = dalloc(&c->G, (size_t)n * n) && dalloc(&c->A0, mm * std::max<int64_t>(c->lda, p)) &&
+  bool ok = dalloc(&c->G, (size_t)n * n) && dalloc(&c->A0, mm * std::max<int64_t>(c->lda, dlk::jau_p4(p))) &&
             dalloc(&c->sidx, mm * s_max) && dalloc(&c->sval, mm * s_max) &&
             dalloc(&c->scnt, mm) && dalloc(&c->bsum, (size_t)2048) &&
             dalloc(&c->err, 1) && dalloc(&c->iter, 1) && dalloc(&c->jw.Upart, nslices * ulen) &&
-            dalloc(&c->jw.U, ulen) && dalloc(&c->jw.Ucopy, ulen * dlk::kUCopies) && dalloc(&c->jw.epart_a, (size_t)2 * c->jw.nb_accum) &&
-            dalloc(&c->jw.epart_b, (size_t)c->jw.nb_row) && dalloc(&c->jw.Dn, (size_t)n * p) &&
+            dalloc(&c->jw.U, ulen) && dalloc(&c->jw.Ucopy, dlk::jau_ulen(dlk::jau_p4(p), n) * dlk::kUCopies) && dalloc(&c->jw.epart_a, (size_t)2 * std::max(c->jw.nb_accum, dlk::jau_plain_blocks(p))) &&
+            dalloc(&c->jw.epart_b, (size_t)c->jw.nb_row) && dalloc(&c->jw.Dn, (size_t)n * dlk::jau_p4(p)) &&
+            dalloc(&c->jw.Dp, (size_t)n * dlk::jau_p4(p)) &&
             dalloc(&c->jw.C, (size_t)n) && dalloc(&c->Dhi, (size_t)n * p) &&
             dalloc(&c->Dlo, (size_t)n * p) && dalloc(&c->rs_list, mm) && dalloc(&c->rs_count, 1);
   ok = ok && cudaStreamCreateWithFlags(&c->st2, cudaStreamNonBlocking) == cudaSuccess &&

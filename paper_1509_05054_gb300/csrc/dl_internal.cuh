@@ -211,7 +211,9 @@ struct JauWork {
   bool copies;      // pass A adds to Ucopy (float4 rows, not deterministic), not to Upart
   double* epart_a;  // [nb_accum][2]  (||E||^2, ||Y||^2) partials
   double* epart_b;  // [nb_row]       ||Y - D'X'||^2 partials
-  float* Dn;        // [n*p] updated atoms
+  float* Dn;        // [n*p] updated atoms (the plain case: rows of jau_p4(p) floats)
+  float* Dp;        // [n*jau_p4(p)] the atoms with padded rows, when padded
+  bool padded;      // the plain case with rows that are not float4 (jau_vec4)
   float* C;         // [n]   d_j^T d_j'
   int nb_accum;
   int nb_row;
@@ -234,7 +236,7 @@ struct JauWork {
   // one slice of Upart each
   bool det = false;
   // the plain case (jau_plain_supported, nb_accum = jau_plain_blocks): the errors
-  // y - D x of all signals (m x p), written by pass A and read by pass B; null otherwise
+  // y - D x of all signals (m x jau_p4(p)), written by pass A and read by pass B; null otherwise
   float* E = nullptr;
 };
 // Grid sizes: mult selects 1x/2x the base CTA count of the accumulation pass
@@ -244,6 +246,7 @@ constexpr int kUCopies = 16;  // copies of U the float4 accumulation spreads its
 // multiple of 4 so that every copy, and with p % 4 == 0 every atom row in it,
 // starts on a 16-byte boundary for the float4 reductions; U and each slice of
 // the partial buffer are allocated with this length.
+__host__ __device__ inline int jau_p4(int p) { return (p + 3) / 4 * 4; }  // padded row length
 __host__ __device__ inline size_t jau_ulen(int p, int n) { return ((size_t)n * p + n + 3) / 4 * 4; }
 int jau_accum_blocks(int p, int n, int mult);
 int jau_accum_blocks_max(int p, int n);
@@ -256,7 +259,7 @@ bool jau_vec4(int p, const float* Y, const float* D);
 // n <= 1024, s <= 16, a range of signals per CTA in shared memory); its CTA count.
 bool jau_det_supported(int p, int n, int s, const float* Y, const float* D);
 int64_t jau_det_ranges(int64_t m, int p, int n, int s);
-bool jau_plain_supported(int64_t m, int p, int n, int s, const float* Y, const float* D);
+bool jau_plain_supported(int64_t m, int p, int n, int s);
 int jau_plain_min();  // fewest signals
 int jau_plain_blocks(int p);
 int jau_plain_row_blocks(int p);

@@ -288,7 +288,10 @@ __global__ void __launch_bounds__(ACC4_THREADS, 4) accum4_kernel(
 }
 
 // ---- The plain case: errors, bucketed sums, rows -------------------------------
-// All atoms at once (no groups, no P-NSGK), float4 rows.  What bounds accum4_kernel
+// All atoms at once (no groups, no P-NSGK).  Rows whose length is no multiple of
+// four floats, or that do not start on 16 bytes, are read float by float from Y; the
+// atoms are then padded once per update (Dp), and E, U and D' have padded rows (p4).
+// What bounds accum4_kernel
 // is the L2's reduction rate: s rows of p floats per signal, 205 MB of vector
 // reductions at p = 64, n = 512, s = 8, m = 1e5 (44.9 us), and what bounds
 // rows4_kernel is issuing about 1,000 instructions per four signals (33.7 us).
@@ -338,6 +341,32 @@ __device__ __forceinline__ void load_once(float4 (&r)[RV], const float4* base, i
     r[q] = on && (FULLP || g + 8 * q < pv) ? ld_once(base + g + 8 * q) : make_float4(0.f, 0.f, 0.f, 0.f);
 }
 
+// Lane g's vectors of the signal at y (p floats): as float4 (YV), or float by float.
+template <int RV, bool FULLP, bool YV>
+__device__ __forceinline__ void load_signal(float4 (&r)[RV], const float* __restrict__ y, int p, int g, int pv,
+                                            bool on) {
+  if constexpr (YV) {
+    load_once<RV, FULLP>(r, (const float4*)y, g, pv, on);
+  } else {
+#pragma unroll
+    for (int q = 0; q < RV; ++q) {
+      const int c = 4 * (g + 8 * q);
+      r[q].x = on && c < p ? __ldg(y + c) : 0.f;
+      r[q].y = on && c + 1 < p ? __ldg(y + c + 1) : 0.f;
+      r[q].z = on && c + 2 < p ? __ldg(y + c + 2) : 0.f;
+      r[q].w = on && c + 3 < p ? __ldg(y + c + 3) : 0.f;
+    }
+  }
+}
+
+// The atoms with rows padded by zeros to p4 floats.
+__global__ void pad_atoms_kernel(const float* __restrict__ D, int p, int n, int p4, float* __restrict__ Dp) {
+  const int q = blockIdx.x * blockDim.x + threadIdx.x;
+  if (q >= n * p4) return;
+  const int j = q / p4, r = q - j * p4;
+  Dp[q] = r < p ? D[(size_t)j * p + r] : 0.f;
+}
+
 // A signal's slots over its eight lanes: lane g holds slots g and g + 8.
 struct Slots {
   int c, j0, j1;
@@ -355,9 +384,10 @@ __device__ __forceinline__ Slots load_slots(int64_t i, bool live, int g, int s, 
   return q;
 }
 
-template <int RV, bool FULLP>
+// D and E have rows of p4 floats.
+template <int RV, bool FULLP, bool YV>
 __global__ void __launch_bounds__(EP_THREADS, RV <= 2 ? 4 : 3) errors_kernel(
-    const float* __restrict__ Y, int p, int64_t m, const float* __restrict__ D, int s,
+    const float* __restrict__ Y, int p, int p4, int64_t m, const float* __restrict__ D, int s,
     const int32_t* __restrict__ idx, const float* __restrict__ val, const int32_t* __restrict__ cnt,
     float* __restrict__ E, double* __restrict__ epart, int* __restrict__ err, float4* __restrict__ Uc,
     int ulen4) {
@@ -366,7 +396,7 @@ __global__ void __launch_bounds__(EP_THREADS, RV <= 2 ? 4 : 3) errors_kernel(
   for (int q = blockIdx.x * EP_THREADS + threadIdx.x; q < ulen4; q += gridDim.x * EP_THREADS)
     Uc[q] = make_float4(0.f, 0.f, 0.f, 0.f);
   const int lane = threadIdx.x & 31, g = lane & 7, gbase = lane & ~7;
-  const int pv = p >> 2;
+  const int pv = p4 >> 2;
   const float4* __restrict__ D4 = (const float4*)D;
   float ee = 0.f, yy = 0.f;
   const int64_t groups = (int64_t)gridDim.x * (EP_THREADS / 8);
@@ -377,7 +407,7 @@ __global__ void __launch_bounds__(EP_THREADS, RV <= 2 ? 4 : 3) errors_kernel(
     const bool live = i < m;
     const Slots sl = next;  // (loaded a trip ahead: the gathers start at once)
     float4 e[RV];
-    load_once<RV, FULLP>(e, (const float4*)Y + (live ? i : 0) * pv, g, pv, live);
+    load_signal<RV, FULLP, YV>(e, Y + (live ? i : 0) * p, p, g, pv, live);
     next = load_slots(i + groups, i + groups < m, g, s, idx, val, cnt);
     const int c = sl.c, o0 = sl.j0 * pv, o1 = sl.j1 * pv;  // row offsets in vectors
     const float x0 = sl.x0, x1 = sl.x1;
@@ -590,16 +620,16 @@ __global__ void __launch_bounds__(SUM_THREADS, 2) sums_kernel(
 
 // Pass B of the plain case: x_t' = e.d'_{j_t} + c_{j_t} x_t (sgk: x_t) into the CSC
 // values, and ||y - D' x'||^2.
-template <int RV, bool FULLP>
+template <int RV, bool FULLP, bool YV>
 __global__ void __launch_bounds__(EP_THREADS, RV <= 1 ? 4 : RV == 2 ? 3 : 2) rows_plain_kernel(
-    const float* __restrict__ Y, const float* __restrict__ E, int p, int64_t m,
+    const float* __restrict__ Y, const float* __restrict__ E, int p, int p4, int64_t m,
     const float* __restrict__ Dn, const float* __restrict__ C, int s, const int32_t* __restrict__ idx,
     const float* __restrict__ val, const int32_t* __restrict__ cnt, const int64_t* __restrict__ colptr,
     float* __restrict__ csc_val, double* __restrict__ epart, int sgk) {
   __shared__ double red[EP_THREADS / 32];
   const int lane = threadIdx.x & 31, g = lane & 7, gbase = lane & ~7;
   const int b2 = g >> 2 & 1, b1 = g >> 1 & 1, tau = 2 * b2 + b1;  // the slot of four this lane sums
-  const int pv = p >> 2;
+  const int pv = p4 >> 2;
   const float4* __restrict__ N4 = (const float4*)Dn;
   float e2 = 0.f;
   const int64_t groups = (int64_t)gridDim.x * (EP_THREADS / 8);
@@ -610,7 +640,7 @@ __global__ void __launch_bounds__(EP_THREADS, RV <= 1 ? 4 : RV == 2 ? 3 : 2) row
     const bool live = i < m;
     const Slots sl = next;
     float4 y[RV], e[RV];
-    load_once<RV, FULLP>(y, (const float4*)Y + (live ? i : 0) * pv, g, pv, live);
+    load_signal<RV, FULLP, YV>(y, Y + (live ? i : 0) * p, p, g, pv, live);
     load_once<RV, FULLP>(e, (const float4*)E + (live ? i : 0) * pv, g, pv, live);
     next = load_slots(i + groups, i + groups < m, g, s, idx, val, cnt);
     const int c = sl.c, j0 = sl.j0, j1 = sl.j1;
@@ -1264,12 +1294,12 @@ constexpr int FIN_THREADS = 128;
 __global__ void __launch_bounds__(FIN_THREADS) finalize_kernel(
     const double* __restrict__ epa, int na, const double* __restrict__ epb, int nb,
     double* __restrict__ rmse, int* __restrict__ iter, const float* __restrict__ Dn,
-    float* __restrict__ D, int64_t np) {
+    float* __restrict__ D, int64_t np, int p, int pitch) {
   __shared__ double red[FIN_THREADS / 32][3];
   if (blockIdx.x > 0) {
     const int64_t stride = (int64_t)(gridDim.x - 1) * blockDim.x;
     for (int64_t q = (int64_t)(blockIdx.x - 1) * blockDim.x + threadIdx.x; q < np; q += stride)
-      D[q] = Dn[q];
+      D[q] = Dn[p == pitch ? q : q / p * pitch + q % p];
     return;
   }
   const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
@@ -1494,7 +1524,7 @@ bool jau_vec4(int p, const float* Y, const float* D) {
 int jau_launches(const JauWork& w) {
   // errors and sums, or one accumulation pass; atoms (after a reduction of the
   // slices where there are no copies); rows; finalize
-  return (w.E ? 2 : 1) + (w.copies ? 1 : 2) + 2;
+  return (w.E ? 2 : 1) + (w.padded ? 1 : 0) + (w.copies ? 1 : 2) + 2;
 }
 int jau_row_blocks(int per_sm) { return (per_sm == 2 || per_sm == 8 ? per_sm : 4) * num_sms(); }
 int jau_row_blocks_max() { return 8 * num_sms(); }
@@ -1503,9 +1533,8 @@ int jau_row_blocks_max() { return 8 * num_sms(); }
 // passes are bound by launches, and accum4_kernel has one launch less (one
 // iteration at p = 16, n = 32, s = 3, m = 1000: 97.4 us against 99.2; p = 64,
 // n = 256, s = 6, m = 20,000: 77.5 against 75.8).
-bool jau_plain_supported(int64_t m, int p, int n, int s, const float* Y, const float* D) {
-  return m >= jau_plain_min() && jau_vec4(p, Y, D) && p <= 128 && n <= 1024 && s <= 16 &&
-         sum_tile(m, p, n, s) > 0;
+bool jau_plain_supported(int64_t m, int p, int n, int s) {
+  return m >= jau_plain_min() && p <= 128 && n <= 1024 && s <= 16 && sum_tile(m, jau_p4(p), n, s) > 0;
 }
 int jau_plain_min() { return 32 * num_sms(); }
 // one full round of resident CTAs each (see the kernels' launch bounds)
@@ -1571,34 +1600,44 @@ cudaError_t jau_accumulate(const float* Y, int p, int64_t m, const float* D, int
                            const JauWork& w, int* err, cudaStream_t st) {
   if (w.det && jau_det_supported(p, n, s, Y, D))
     return jau_accumulate_det(Y, p, m, D, n, s, idx, val, cnt, w, err, st);
+  if (w.E) {  // the plain case
+    const int p4 = jau_p4(p);
+    const size_t len = jau_ulen(p4, n);
+    const bool vec = jau_vec4(p, Y, D);
+    cudaError_t e;
+    if (!vec) {
+      pad_atoms_kernel<<<(n * p4 + 255) / 256, 256, 0, st>>>(D, p, n, p4, w.Dp);
+      if ((e = cudaGetLastError()) != cudaSuccess) return e;
+    }
+#define DL_ERRS(RV)                                                                                  \
+  do {                                                                                               \
+    auto kern = !vec ? errors_kernel<RV, false, false>                                               \
+                     : p == 32 * RV ? errors_kernel<RV, true, true> : errors_kernel<RV, false, true>; \
+    cudaFuncSetAttribute(kern, cudaFuncAttributePreferredSharedMemoryCarveout,                       \
+                         cudaSharedmemCarveoutMaxL1);                                                \
+    kern<<<w.nb_accum, EP_THREADS, 0, st>>>(Y, p, p4, m, vec ? D : w.Dp, s, idx, val, cnt, w.E,      \
+                                            w.epart_a, err, (float4*)w.Ucopy,                        \
+                                            (int)(len * kUCopies / 4));                              \
+  } while (0)
+    if (p <= 32) DL_ERRS(1);
+    else if (p <= 64) DL_ERRS(2);
+    else if (p <= 96) DL_ERRS(3);
+    else DL_ERRS(4);
+#undef DL_ERRS
+    if ((e = cudaGetLastError()) != cudaSuccess) return e;
+    const int T = sum_tile(m, p4, n, s);
+    const size_t smem = (size_t)SumSmem(p4, n, s, T).total;
+    if ((e = cudaFuncSetAttribute(sums_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem)) !=
+        cudaSuccess)
+      return e;
+    const int64_t nt = (m + T - 1) / T;
+    sums_kernel<<<(unsigned)(nt < 2 * num_sms() ? nt : 2 * num_sms()), SUM_THREADS, smem, st>>>(
+        w.E, p4, m, T, n, s, idx, val, w.Ucopy, err);
+    return cudaGetLastError();
+  }
   if (jau_vec4(p, Y, D)) {
     const size_t len = jau_ulen(p, n);
-    cudaError_t e = cudaSuccess;
-    if (w.E) {  // the plain case
-#define DL_ERRS(RV)                                                                              \
-  do {                                                                                           \
-    auto kern = p == 32 * RV ? errors_kernel<RV, true> : errors_kernel<RV, false>;               \
-    cudaFuncSetAttribute(kern, cudaFuncAttributePreferredSharedMemoryCarveout,                   \
-                         cudaSharedmemCarveoutMaxL1);                                            \
-    kern<<<w.nb_accum, EP_THREADS, 0, st>>>(Y, p, m, D, s, idx, val, cnt, w.E, w.epart_a, err,   \
-                                            (float4*)w.Ucopy, (int)(len * kUCopies / 4));        \
-  } while (0)
-      if (p <= 32) DL_ERRS(1);
-      else if (p <= 64) DL_ERRS(2);
-      else if (p <= 96) DL_ERRS(3);
-      else DL_ERRS(4);
-#undef DL_ERRS
-      if ((e = cudaGetLastError()) != cudaSuccess) return e;
-      const int T = sum_tile(m, p, n, s);
-      const size_t smem = (size_t)SumSmem(p, n, s, T).total;
-      if ((e = cudaFuncSetAttribute(sums_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                    (int)smem)) != cudaSuccess)
-        return e;
-      const int64_t nt = (m + T - 1) / T;
-      sums_kernel<<<(unsigned)(nt < 2 * num_sms() ? nt : 2 * num_sms()), SUM_THREADS, smem, st>>>(
-          w.E, p, m, T, n, s, idx, val, w.Ucopy, err);
-      return cudaGetLastError();
-    }
+    cudaError_t e;
     if ((e = cudaMemsetAsync(w.Ucopy, 0, sizeof(float) * len * kUCopies, st)) != cudaSuccess) return e;
 #define DL_ACC4(RV, SM)                                                                  \
   do {                                                                                       \
@@ -1648,7 +1687,8 @@ cudaError_t jau_accumulate(const float* Y, int p, int64_t m, const float* D, int
 cudaError_t jau_atoms(const float* D, int p, int n, const JauWork& w, cudaStream_t st) {
   const int a0 = w.a0, a1 = w.a1 > 0 ? w.a1 : n;
   if (w.copies) {
-    if (a1 > a0) atoms4_kernel<<<a1 - a0, 256, 0, st>>>(D, p, n, w.Ucopy, w.Dn, w.C, a0);
+    if (a1 > a0)
+      atoms4_kernel<<<a1 - a0, 256, 0, st>>>(w.padded ? w.Dp : D, jau_p4(p), n, w.Ucopy, w.Dn, w.C, a0);
     return cudaGetLastError();
   }
   const int blocks = (a1 - a0 + 7) / 8;
@@ -1669,13 +1709,17 @@ cudaError_t jau_rows(const float* Y, int p, int64_t m, const float* D, int n, in
 #define DL_ROWS(PL)                                                                              \
   rows_kernel<PL><<<nb, ROW_THREADS, 0, st>>>(Y, p, m, D, w.Dn, w.C, s, idx, val, cnt, colptr, \
                                               csc_rowidx, csc_val, w.epart_b, (int)w.sgk)
-  if (w.E && !csc_rowidx) {  // the plain case
+  if (w.E) {  // the plain case (the row indices are the coding pass's: csc_rowidx is null)
+    const int p4 = jau_p4(p);
+    const bool vec = jau_vec4(p, Y, D);
 #define DL_ROWSP(RV)                                                                              \
   do {                                                                                            \
-    auto kern = p == 32 * RV ? rows_plain_kernel<RV, true> : rows_plain_kernel<RV, false>;        \
+    auto kern = !vec ? rows_plain_kernel<RV, false, false>                                        \
+                     : p == 32 * RV ? rows_plain_kernel<RV, true, true>                           \
+                                    : rows_plain_kernel<RV, false, true>;                         \
     cudaFuncSetAttribute(kern, cudaFuncAttributePreferredSharedMemoryCarveout,                    \
                          cudaSharedmemCarveoutMaxL1);                                             \
-    kern<<<nb, EP_THREADS, 0, st>>>(Y, w.E, p, m, w.Dn, w.C, s, idx, val, cnt, colptr, csc_val,   \
+    kern<<<nb, EP_THREADS, 0, st>>>(Y, w.E, p, p4, m, w.Dn, w.C, s, idx, val, cnt, colptr, csc_val, \
                                     w.epart_b, (int)w.sgk);                                       \
   } while (0)
     if (p <= 32) DL_ROWSP(1);
@@ -1722,7 +1766,8 @@ cudaError_t jau_finalize(const JauWork& w, double* rmse_out, int* iter, float* D
   int64_t cb = (np + FIN_THREADS - 1) / FIN_THREADS;
   if (cb > 256) cb = 256;
   finalize_kernel<<<(unsigned)(1 + cb), FIN_THREADS, 0, st>>>(w.epart_a, w.nb_accum, w.epart_b,
-                                                              w.nb_row, rmse_out, iter, w.Dn, D, np);
+                                                              w.nb_row, rmse_out, iter, w.Dn, D, np, p,
+                                                              w.E ? jau_p4(p) : p);
   return cudaGetLastError();
 }
 
