@@ -112,6 +112,8 @@ struct Shape {
   static constexpr int W = 4 * Q;
   static constexpr int NTM = (512 / Q) / NT < DL_RESOLVE_SMAX - 1 ? (512 / Q) / NT : DL_RESOLVE_SMAX - 1;
   static constexpr int COLS = NTM * NT;
+  // registers for two vectors of TMEM loads in flight (65536 / threads, less the rest)
+  static constexpr bool TWO = 512 / Q - 64 >= 3 * NT;
   static_assert(COLS * Q <= 512 && NTM >= 1, "TMEM columns");
   // dynamic shared memory for supports of s: vectors past NTM, and the Cholesky rows
   static size_t smem(int s) {
@@ -123,7 +125,7 @@ struct Shape {
 // The OMP of signal i by one warp; see omp_one (omp_one.cuh) for the steps.
 // tcol: TMEM address of this warp's first column; u_q for q < NTM at tcol +
 // NT q, the others in u_s (shared memory, [q - NTM][pair][lane]); L: s x s.
-template <int NT, int NTM, bool FULLN>
+template <int NT, int NTM, bool FULLN, bool TWO>
 __device__ __forceinline__ void omp_one_roll(
     int64_t i, const float* __restrict__ G, int n, float* L, float2* u_s, uint32_t tcol,
     const float* __restrict__ a0row, const float* __restrict__ y, int p, int s,
@@ -255,14 +257,8 @@ __device__ __forceinline__ void omp_one_roll(
 
     if (need_u) {  // u_step = G[:, sel] + sum_q negaw_q u_q;  alpha -= (z_k c_k) u_step
       const int nt = step < NTM ? step : NTM;
-#pragma unroll 1
-      for (int q = 0; q < nt; ++q) {
-        const float nq = __shfl_sync(FULL, negaw, q);
+      auto add = [&](float nq, uint32_t (&r)[NT / C][C]) {
         const float2 nw = make_float2(nq, nq);
-        uint32_t r[NT / C][C];
-#pragma unroll
-        for (int h = 0; h < NT / C; ++h) tm_ld(tcol + NT * q + C * h, r[h]);
-        tm_wait();
 #pragma unroll
         for (int h = 0; h < NT / C; ++h) {
           tie(r[h]);
@@ -272,8 +268,32 @@ __device__ __forceinline__ void omp_one_roll(
             gv = __ffma2_rn(nw, make_float2(__uint_as_float(r[h][2 * v]), __uint_as_float(r[h][2 * v + 1])), gv);
           }
         }
+      };
+      int q0 = 0;
+      if constexpr (TWO) {  // two vectors per wait, while the registers allow it
+#pragma unroll 1
+        for (; q0 + 1 < nt; q0 += 2) {
+          uint32_t r0[NT / C][C], r1[NT / C][C];
+#pragma unroll
+          for (int h = 0; h < NT / C; ++h) tm_ld(tcol + NT * q0 + C * h, r0[h]);
+#pragma unroll
+          for (int h = 0; h < NT / C; ++h) tm_ld(tcol + NT * (q0 + 1) + C * h, r1[h]);
+          const float n0 = __shfl_sync(FULL, negaw, q0), n1 = __shfl_sync(FULL, negaw, q0 + 1);
+          tm_wait();
+          add(n0, r0);
+          add(n1, r1);
+        }
       }
 #pragma unroll 1
+      for (int q = q0; q < nt; ++q) {
+        uint32_t r[NT / C][C];
+#pragma unroll
+        for (int h = 0; h < NT / C; ++h) tm_ld(tcol + NT * q + C * h, r[h]);
+        const float nq = __shfl_sync(FULL, negaw, q);
+        tm_wait();
+        add(nq, r);
+      }
+#pragma unroll 2
       for (int q = NTM; q < step; ++q) {
         const float nq = __shfl_sync(FULL, negaw, q);
         const float2 nw = make_float2(nq, nq);
@@ -370,7 +390,7 @@ __global__ void __launch_bounds__(Q * 128, 1) omp_roll_kernel(
       if (lane * 32 < n) asm volatile("prefetch.global.L2 [%0];" ::"l"(A0 + ip * lda + lane * 32));
       if (lane * 32 < p) asm volatile("prefetch.global.L2 [%0];" ::"l"(Y + ip * p + lane * 32));
     }
-    omp_one_roll<NT, S::NTM, FULLN>(i, G, n, L, u_s, tcol, A0 + i * lda, Y + i * p, p, s, oidx, oval,
+    omp_one_roll<NT, S::NTM, FULLN, S::TWO>(i, G, n, L, u_s, tcol, A0 + i * lda, Y + i * p, p, s, oidx, oval,
                                     ocnt, ores, err, rs_list, rs_count, rs_cap, gap_tol);
   }
   tc::tc_fence_before();
