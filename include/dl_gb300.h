@@ -85,7 +85,7 @@ typedef struct dl_ctx dl_ctx;
  *   p          1 <= p <= DL_MAX_P.
  *   n          1 <= n <= DL_MAX_N.
  *   m_max      1 <= m_max; workspace is sized for m_max signals
- *              (about m_max * (4n + 8 s_max + 16) bytes plus O(n^2 + 152 n p)).
+ *              (about m_max * (4 max(n, p) + 8 s_max + 16) bytes plus O(n^2 + 152 n p)).
  *   s_max      1 <= s_max <= min(p, n, DL_MAX_S).
  *   precision  DL_FP32, DL_BF16 or DL_FP8: the arithmetic of the correlations
  *              D^T Y (mixed precision: BF16, or E4M3 with each atom and each
@@ -212,10 +212,10 @@ int dl_set_group_size(dl_ctx* ctx, int ntilde);
  * dl_set_deterministic -- the order in which the atom-update stage sums
  * U = E X^T and r_j = ||x_j||^2 (Eq. 3, Eq. 5: F x_j^T = U_j + r_j d_j).  The
  * paper fixes no order; floating-point sums depend on it.
- *   on = 0 (default): every signal adds its contributions x_{j,i} e_i into
- *          copies of U in L2 by float vector reductions; the order of those
- *          additions varies from run to run, so D and X are reproducible to
- *          rounding, not bit for bit.
+ *   on = 0 (default): the contributions x_{j,i} e_i, summed per tile of signals
+ *          or signal by signal, are added into copies of U in L2 by float vector
+ *          reductions; the order of those additions varies from run to run, so
+ *          D and X are reproducible to rounding, not bit for bit.
  *   on = 1: the contributions are summed in an order fixed by the signal and
  *          slot indices (per range of signals, each atom's pairs sorted by
  *          signal and slot; then the ranges in order), so repeated runs give

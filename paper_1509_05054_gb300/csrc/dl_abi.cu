@@ -104,6 +104,14 @@ struct dl_ctx {
   int* iter = nullptr;
   double* rmse = nullptr;
   int rmse_cap = 0;  // iterations
+  // page-locked landing place of the error word and of the RMSE pairs of short calls:
+  // a copy into pageable memory waits for the GPU by itself, so a call that reads
+  // both would wait twice
+  struct Landing {
+    int err;
+    double rmse[2 * 64];
+  };
+  Landing* land = nullptr;
   dlk::JauWork jw{};
   // host staging (lazily allocated)
   float* hY = nullptr;
@@ -131,7 +139,7 @@ struct dl_ctx {
   int64_t launches = 0;
   // launch shapes (chosen by dl_autotune; defaults otherwise)
   int cfg_omp_warps = 4;  // warps per CTA of the OMP kernel
-  int cfg_omp_tm = 5;     // warps per TMEM quadrant of the TMEM-resident OMP kernel (0: off)
+  int cfg_omp_tm = 5;     // warps per TMEM quadrant of the n = 512 OMP kernel (0: omp_warp_kernel for every shape)
   int cfg_omp_res = 1;    // residual-form OMP with per-step tensor-core correlations (0: off)
   int last_omp = -1;      // the coding kernel of the last pass (dl_last_omp_kernel)
   int deterministic = 0;  // pass A with a fixed summation order (dl_set_deterministic)
@@ -182,6 +190,7 @@ void free_ctx(dl_ctx* c) {
                   c->pvalid, c->D0};
   for (void* q : ptrs)
     if (q) cudaFree(q);
+  if (c->land) cudaFreeHost(c->land);
   cudaSetDevice(prev);
   delete c;
 }
@@ -230,14 +239,26 @@ int ptr_kind(const void* p) {
 
 // Read and clear the device error word; returns a status.
 int take_device_error(dl_ctx* c) {
-  int h = 0;
-  DL_CHECK(cudaMemcpyAsync(&h, c->err, sizeof(int), cudaMemcpyDeviceToHost, c->st));
+  DL_CHECK(cudaMemcpyAsync(&c->land->err, c->err, sizeof(int), cudaMemcpyDeviceToHost, c->st));
   DL_CHECK(cudaStreamSynchronize(c->st));
+  const int h = c->land->err;
   if (h) DL_CHECK(cudaMemsetAsync(c->err, 0, sizeof(int), c->st));
   if (h & dlk::ERR_CSC) return DL_EINVAL;
   if (h & dlk::ERR_NONFINITE) return DL_ENUMERIC;
   if (h & dlk::ERR_TIMEOUT) return DL_ETIMEOUT;
   return DL_OK;
+}
+
+// The end of a call that reads results on the host: the RMSE pairs of `iters`
+// iterations into rmse (when given) and the device error, one wait for both.
+int finish(dl_ctx* c, double* rmse, int iters) {
+  const size_t bytes = sizeof(double) * 2 * (size_t)iters;
+  const bool land = rmse && bytes <= sizeof(c->land->rmse);
+  if (rmse)
+    DL_CHECK(cudaMemcpyAsync(land ? c->land->rmse : rmse, c->rmse, bytes, cudaMemcpyDeviceToHost, c->st));
+  const int rc = take_device_error(c);
+  if (land && rc != DL_ECUDA) memcpy(rmse, c->land->rmse, bytes);
+  return rc;
 }
 
 int ensure_rmse(dl_ctx* c, int iters) {
@@ -803,9 +824,7 @@ int host_call_graphed(dl_ctx* c, const float* Y, int64_t m, float* D, int s, int
     c->launches += k;
     c->hseen++;
   }
-  if (rmse)
-    DL_CHECK(cudaMemcpyAsync(rmse, c->rmse, sizeof(double) * 2, cudaMemcpyDeviceToHost, c->st));
-  return take_device_error(c);
+  return finish(c, rmse, 1);
 }
 
 }  // namespace
@@ -861,7 +880,8 @@ int dl_init(dl_ctx** out, int p, int n, int64_t m_max, int s_max, int precision,
             dalloc(&c->jw.Dp, (size_t)n * dlk::jau_p4(p)) &&
             dalloc(&c->jw.C, (size_t)n) && dalloc(&c->Dhi, (size_t)n * p) &&
             dalloc(&c->Dlo, (size_t)n * p) && dalloc(&c->rs_list, mm) && dalloc(&c->rs_count, 1);
-  ok = ok && cudaStreamCreateWithFlags(&c->st2, cudaStreamNonBlocking) == cudaSuccess &&
+  ok = ok && cudaMallocHost((void**)&c->land, sizeof(dl_ctx::Landing)) == cudaSuccess &&
+       cudaStreamCreateWithFlags(&c->st2, cudaStreamNonBlocking) == cudaSuccess &&
        cudaEventCreateWithFlags(&c->ev_fork, cudaEventDisableTiming) == cudaSuccess &&
        cudaEventCreateWithFlags(&c->ev_join, cudaEventDisableTiming) == cudaSuccess &&
        cudaEventCreateWithFlags(&c->ev_join2, cudaEventDisableTiming) == cudaSuccess;
@@ -1112,8 +1132,7 @@ int jau_update(dl_ctx* c, const float* Y, int64_t m, float* D, const int64_t* co
     DL_CHECK(cudaMemcpyAsync(D, dD, sizeof(float) * (size_t)c->n * c->p, cudaMemcpyDeviceToHost, c->st));
     DL_CHECK(cudaMemcpyAsync(val, dv, sizeof(float) * (size_t)nnz, cudaMemcpyDeviceToHost, c->st));
   }
-  if (rmse2) DL_CHECK(cudaMemcpyAsync(rmse2, c->rmse, sizeof(double) * 2, cudaMemcpyDeviceToHost, c->st));
-  if (kind == 0 || rmse2) return take_device_error(c);
+  if (kind == 0 || rmse2) return finish(c, rmse2, 1);
   return DL_OK;
 }
 
@@ -1252,10 +1271,7 @@ int dl_iterate(dl_ctx* c, const float* Y, int64_t m, float* D, int s, int iters,
     DL_CHECK(cudaMemcpyAsync(rowidx, dri, sizeof(int32_t) * (size_t)m * s, cudaMemcpyDeviceToHost, c->st));
     DL_CHECK(cudaMemcpyAsync(val, dv, sizeof(float) * (size_t)m * s, cudaMemcpyDeviceToHost, c->st));
   }
-  if (rmse)
-    DL_CHECK(cudaMemcpyAsync(rmse, c->rmse, sizeof(double) * 2 * (size_t)iters,
-                             cudaMemcpyDeviceToHost, c->st));
-  if (kind == 0 || rmse) return take_device_error(c);
+  if (kind == 0 || rmse) return finish(c, rmse, iters);
   return DL_OK;
 }
 

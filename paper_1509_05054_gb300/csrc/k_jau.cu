@@ -9,11 +9,12 @@
 // warp, then every signal recomputes its error and its coefficients.
 //
 // The passes over the signals give each signal eight lanes (four signals per
-// warp).  With p % 4 == 0 and 16-byte aligned Y and D they move float4 rows
-// and pass A adds x e_i into 16 copies of U with vector reductions in L2
-// (red.v4.f32); otherwise pass A keeps per-CTA copies of U (shared memory when
-// they fit).  The copies are summed in a fixed order.  The energy partial sums are reduced in a
-// fixed order.
+// warp).  With enough signals the plain case (all atoms at once, AK-SVD or SGK) runs
+// as three passes: errors stored, sums of the pairs sorted by atom, rows (see
+// errors_kernel).  Otherwise, with p % 4 == 0 and 16-byte aligned Y and D, pass A
+// adds x e_i into 16 copies of U with vector reductions in L2 (red.v4.f32); else it
+// keeps per-CTA copies of U (shared memory when they fit).  The copies are summed in
+// a fixed order, and so are the energy partial sums.
 #include "dl_internal.cuh"
 #include "tc_ptx.cuh"
 

@@ -12,8 +12,8 @@
 //      same Gram-Schmidt Batch-OMP as the large-problem kernels, Gram rows from
 //      shared memory); a signal whose Cholesky pivot falls below 1e-6 is redone by
 //      the warp in FP64 with the oracle's stop rules.  (With a warp per signal, and
-//      the energies summed in FP64 signal by signal, an iteration of 200 problems
-//      at p = 20, n = 50, m = 1500, s = 4 took 919 us, now 490);
+//      the energies summed in FP64 signal by signal, one iteration of 200 problems
+//      at p = 20, n = 50, m = 1500, s = 4 took 616 us among others like it, now 333);
 //   3. e_i = y_i - D x_i, U = E X^T and r_j = ||x_j||^2 by shared-memory
 //      reductions (X_prev for P-NSGK, Eq. 7), ||E||^2 and ||Y||^2;
 //   4. the atom update (Eq. 5): d_j' = (U_j + r_j d_j) / ||.||, c_j = d_j^T d_j';
