@@ -134,6 +134,7 @@ __device__ __forceinline__ void omp_sub_core(int64_t i, bool live, float4 (&a)[V
     float ck = rsqrtf(delta);
     ck = fmaf(0.5f * ck, fmaf(-delta * ck, ck, 1.0f), ck);
     const float zk = asel * ck;
+    __syncwarp();  // every lane has read the selected atom's four correlations
     if (act) {
       if (l == step) {
         myc = ck;
