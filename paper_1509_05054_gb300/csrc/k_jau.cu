@@ -1331,7 +1331,8 @@ __global__ void __launch_bounds__(FIN_THREADS) finalize_kernel(
     yy += red[q][1];
     e2 += red[q][2];
   }
-  const int it = *iter;
+  // (one lane reads and advances the counter: the other lanes never see it move)
+  const int it = __shfl_sync(FULL, lane == 0 ? *iter : 0, 0);
   if (lane < 2) {
     const double num = lane == 0 ? ee : e2;
     rmse[2 * it + lane] = yy > 0.0 ? sqrt(num / yy) : 0.0;
