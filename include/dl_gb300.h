@@ -349,7 +349,8 @@ int dl_get_config(dl_ctx* ctx, int* cfg4);
  * dl_last_omp_kernel -- which sparse-coding kernel the context's last coding
  * pass (omp_code, dl_iterate) ran (Algorithm 1 step 1), one of
  *   0  Batch-OMP from stored correlations alpha0, one or several signals per warp
- *   1  the same with the progressive-Cholesky vectors in TMEM
+ *   1  the same with the progressive-Cholesky vectors in TMEM, or, for supports
+ *      past 8 and n > 512 in calls of few signals, in shared memory
  *   2  residual-form OMP, the correlations D^T r of every step on the tensor
  *      cores (FP16 hi/lo parts, or BF16 operands in the DL_BF16 form; FP32
  *      accumulation), no stored alpha0; taken for FP32 and BF16 calls without

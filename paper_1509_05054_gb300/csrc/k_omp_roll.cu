@@ -106,19 +106,19 @@ __device__ __forceinline__ float take_alpha(float2 (&alpha)[NT / 2], int tsel, f
   return out;
 }
 
-// Columns of TMEM and vectors in TMEM of each of 4Q warps.
-template <int NT, int Q>
+// Columns of TMEM and vectors in TMEM of each of 4Q warps (TM; none otherwise).
+template <int NT, int Q, bool TM>
 struct Shape {
   static constexpr int W = 4 * Q;
-  static constexpr int NTM = (512 / Q) / NT < DL_RESOLVE_SMAX - 1 ? (512 / Q) / NT : DL_RESOLVE_SMAX - 1;
+  static constexpr int NTM = !TM ? 0 : (512 / Q) / NT < DL_RESOLVE_SMAX - 1 ? (512 / Q) / NT : DL_RESOLVE_SMAX - 1;
   static constexpr int COLS = NTM * NT;
   // registers for two vectors of TMEM loads in flight (65536 / threads, less the rest)
   static constexpr bool TWO = 512 / Q - 64 >= 3 * NT;
-  static_assert(COLS * Q <= 512 && NTM >= 1, "TMEM columns");
-  // dynamic shared memory for supports of s: vectors past NTM, and the Cholesky rows
-  static size_t smem(int s) {
+  static_assert(COLS * Q <= 512 && (NTM >= 1 || !TM), "TMEM columns");
+  // dynamic shared memory of `warps` warps for supports of s: vectors past NTM, and the Cholesky rows
+  static size_t smem(int s, int warps = W) {
     const int nsh = s - 1 > NTM ? s - 1 - NTM : 0;
-    return (size_t)W * ((size_t)nsh * NT * 32 * sizeof(float) + (size_t)s * s * sizeof(float));
+    return (size_t)warps * ((size_t)nsh * NT * 32 * sizeof(float) + (size_t)s * s * sizeof(float));
   }
 };
 
@@ -190,17 +190,19 @@ __device__ __forceinline__ void omp_one_roll(
     // owning lane, or the owning lane's entry in shared memory
     float ul = 0.f;
     {
-      uint32_t tv[NTM];
-      if (step > 0) tm_wait_st();  // u_{step-1} was just stored
+      if constexpr (NTM > 0) {
+        uint32_t tv[NTM];
+        if (step > 0) tm_wait_st();  // u_{step-1} was just stored
 #pragma unroll
-      for (int q = 0; q < NTM; ++q) tv[q] = q < step ? tm_ld1(tcol + NT * q + tsel) : 0u;
-      tm_wait();
-      tie(tv);
+        for (int q = 0; q < NTM; ++q) tv[q] = q < step ? tm_ld1(tcol + NT * q + tsel) : 0u;
+        tm_wait();
+        tie(tv);
 #pragma unroll
-      for (int q = 0; q < NTM; ++q) {
-        if (q >= step) break;
-        const float v = __shfl_sync(FULL, __uint_as_float(tv[q]), lsel);
-        if (lane == q) ul = v;
+        for (int q = 0; q < NTM; ++q) {
+          if (q >= step) break;
+          const float v = __shfl_sync(FULL, __uint_as_float(tv[q]), lsel);
+          if (lane == q) ul = v;
+        }
       }
       if (lane >= NTM && lane < step) {
         const float2 pr = u_s[((lane - NTM) * NV + (tsel >> 1)) * 32 + lsel];
@@ -325,7 +327,7 @@ __device__ __forceinline__ void omp_one_roll(
     __syncwarp();  // row `step` of L and a shared u_step are read later
     if (rr <= kResidRel * yy) break;
   }
-  tm_wait_st();
+  if constexpr (NTM > 0) tm_wait_st();
   __syncwarp();
 
   // ---- back substitution L^T gamma = z
@@ -354,31 +356,34 @@ __device__ __forceinline__ void omp_one_roll(
   __syncwarp();
 }
 
-// Persistent: one CTA of 4Q warps per SM; warp w of CTA b codes signals
-// b * 4Q + w + t * gridDim.x * 4Q.
-template <int NT, int Q, bool FULLN>
+// Persistent: one CTA of W <= 4Q warps per SM; warp w of CTA b codes signals
+// b * W + w + t * gridDim.x * W.
+template <int NT, int Q, bool TM, bool FULLN>
 __global__ void __launch_bounds__(Q * 128, 1) omp_roll_kernel(
     const float* __restrict__ A0, int64_t lda, const float* __restrict__ G, int n,
     const float* __restrict__ Y, int p, int64_t m, int s, int32_t* __restrict__ oidx,
     float* __restrict__ oval, int32_t* __restrict__ ocnt, float* __restrict__ ores,
     int* __restrict__ err, int* __restrict__ rs_list, int* __restrict__ rs_count, int rs_cap,
     float gap_tol) {
-  using S = Shape<NT, Q>;
-  constexpr int W = S::W;
+  using S = Shape<NT, Q, TM>;
+  const int W = blockDim.x >> 5;
   extern __shared__ float2 smem_u[];
   __shared__ uint32_t tbase_sh;
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-  if (warp == 0) {
+  if (TM && warp == 0) {
     asm volatile("tcgen05.alloc.cta_group::1.sync.aligned.shared::cta.b32 [%0], %1;" ::"r"(
                      tc::smem_u32(&tbase_sh)),
                  "r"(512)
                  : "memory");
     asm volatile("tcgen05.relinquish_alloc_permit.cta_group::1.sync.aligned;" ::: "memory");
   }
-  tc::tc_fence_before();
-  __syncthreads();
-  tc::tc_fence_after();
-  const uint32_t tbase = tbase_sh;
+  uint32_t tbase = 0;
+  if (TM) {
+    tc::tc_fence_before();
+    __syncthreads();
+    tc::tc_fence_after();
+    tbase = tbase_sh;
+  }
   const uint32_t tcol = tbase + ((uint32_t)(32 * (warp & 3)) << 16) + (uint32_t)((warp >> 2) * S::COLS);
   const int nsh = s - 1 > S::NTM ? s - 1 - S::NTM : 0;
   float2* u_s = smem_u + (size_t)warp * nsh * (NT / 2) * 32;
@@ -393,6 +398,7 @@ __global__ void __launch_bounds__(Q * 128, 1) omp_roll_kernel(
     omp_one_roll<NT, S::NTM, FULLN, S::TWO>(i, G, n, L, u_s, tcol, A0 + i * lda, Y + i * p, p, s, oidx, oval,
                                     ocnt, ores, err, rs_list, rs_count, rs_cap, gap_tol);
   }
+  if (!TM) return;
   tc::tc_fence_before();
   __syncthreads();
   if (warp == 0)
@@ -402,15 +408,19 @@ __global__ void __launch_bounds__(Q * 128, 1) omp_roll_kernel(
 
 constexpr size_t kRollSmem = 226 * 1024;  // dynamic shared memory one CTA may ask for
 
-template <int NT, int Q>
+template <int NT, int Q, bool TM>
 cudaError_t launch_q(const float* A0, int64_t lda, const float* G, int n, const float* Y, int p,
                      int64_t m, int s, int32_t* idx, float* val, int32_t* cnt, float* ores,
                      int* err, int* rl, int* rc, int rcap, float gt, cudaStream_t st) {
-  const size_t smem = Shape<NT, Q>::smem(s);
-  auto kern = n == 32 * NT ? omp_roll_kernel<NT, Q, true> : omp_roll_kernel<NT, Q, false>;
+  // the rounds that 4Q warps per SM need, with the signals spread evenly over them:
+  // no warp more than that
+  const int64_t round = (int64_t)num_sms() * Shape<NT, Q, TM>::W;
+  const int64_t slots = (m + round - 1) / round * num_sms();
+  const int W = (int)((m + slots - 1) / slots);
+  const size_t smem = Shape<NT, Q, TM>::smem(s, W);
+  auto kern = n == 32 * NT ? omp_roll_kernel<NT, Q, TM, true> : omp_roll_kernel<NT, Q, TM, false>;
   cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
   if (e != cudaSuccess) return e;
-  constexpr int W = Shape<NT, Q>::W;
   const int64_t need = (m + W - 1) / W;
   const int grid = (int)(need < num_sms() ? need : num_sms());
   kern<<<grid, W * 32, smem, st>>>(A0, lda, G, n, Y, p, m, s, idx, val, cnt, ores, err, rl, rc, rcap, gt);
@@ -425,6 +435,14 @@ cudaError_t launch_q(const float* A0, int64_t lda, const float* G, int n, const 
 // in registers, 62 against 49), and supports past 8 (m = 40,000: n = 512, s = 9
 // 177 against 215 us, s = 16 577 against 821; n = 256, s = 10 165 against 235).
 // With s <= 8 and n <= 512 the unrolled kernels are as fast or faster.
+//
+// A call of few signals is one round of at most a few warps per SM, and its time is
+// one signal's chain of steps, of which TMEM's latency is a large part: while
+// the vectors of the warps of that one round fit in shared memory, they all lie there
+// and no TMEM is allocated.  n = 256, s = 10, m = 300 9.2 us (in TMEM with the
+// signals on as few SMs as hold them 20.8, spread over all SMs 12.6; omp_warp_kernel
+// 7.9); n = 512, s = 12, m = 600 12.9 (23.2, 16.5; 13.4); n = 1024, s = 10, m = 600
+// 13.0 (19.4, 14.9; 27).
 bool omp_roll_supported(int n, int s) {
   return n > 128 && n <= 1024 && s <= DL_RESOLVE_SMAX && (s > 8 || (n > 512 && s > 4));
 }
@@ -434,25 +452,33 @@ cudaError_t omp_roll(const float* A0, int64_t lda, const float* G, int n, const 
                      int* err, int* rl, int* rc, int rcap, float gt, cudaStream_t st) {
   if (!omp_roll_supported(n, s)) return cudaErrorInvalidValue;
   if (m <= 0) return cudaSuccess;
-  // the most warps whose vectors fit
-#define DL_ROLL(NT, Q)                     \
-  if (Shape<NT, Q>::smem(s) <= kRollSmem) \
-  return launch_q<NT, Q>(A0, lda, G, n, Y, p, m, s, idx, val, cnt, ores, err, rl, rc, rcap, gt, st)
+  // one round with every vector in shared memory, else the most warps whose vectors fit
+#define DL_ROLL_SH(NT, Q)                                                                 \
+  if (m <= 4 * Q * (int64_t)num_sms() &&                                                  \
+      Shape<NT, Q, false>::smem(s, (int)((m + num_sms() - 1) / num_sms())) <= kRollSmem)  \
+  return launch_q<NT, Q, false>(A0, lda, G, n, Y, p, m, s, idx, val, cnt, ores, err, rl, rc, rcap, gt, st)
+#define DL_ROLL(NT, Q)                          \
+  if (Shape<NT, Q, true>::smem(s) <= kRollSmem) \
+  return launch_q<NT, Q, true>(A0, lda, G, n, Y, p, m, s, idx, val, cnt, ores, err, rl, rc, rcap, gt, st)
   if (n > 512) {
+    DL_ROLL_SH(32, 2);
     DL_ROLL(32, 4);
     DL_ROLL(32, 3);
     DL_ROLL(32, 2);
     DL_ROLL(32, 1);
   } else if (n > 256) {
+    DL_ROLL_SH(16, 4);
     DL_ROLL(16, 6);
     DL_ROLL(16, 5);
     DL_ROLL(16, 4);
     DL_ROLL(16, 3);
   } else {
+    DL_ROLL_SH(8, 4);
     DL_ROLL(8, 8);
     DL_ROLL(8, 6);
   }
 #undef DL_ROLL
+#undef DL_ROLL_SH
   return cudaErrorInvalidValue;
 }
 
