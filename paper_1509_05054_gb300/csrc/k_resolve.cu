@@ -5,9 +5,11 @@
 // decision and the coefficients are those of the FP64 Batch-OMP:
 //
 //   * the residual r = y - D_I gamma is kept in FP64 (p values), with gamma from
-//     the FP64 inverse Cholesky factor B of G[I,I] (entries d_q^T d_sel taken in
-//     FP64 from the FP32 atoms, which FP64 holds exactly): w = B g, the new row
-//     of B from w, gamma += z B_k;
+//     the FP64 Cholesky factor L of G[I,I] (entries d_q^T d_sel taken in FP64 from
+//     the FP32 atoms, which FP64 holds exactly) by triangular solves, L z = D_I^T y
+//     and L^T gamma = z.  (Kept as an inverse factor, gamma += z B_k, the
+//     coefficients of eight near-dependent atoms with a pivot of 2e-9 were off by 1e-4
+//     of the largest; solves leave 5e-7, the error of FP64 Cholesky itself.)
 //   * each step's correlations alpha = alpha0 - G[:, I] gamma are taken in
 //     FP32, fresh every step (no rounding carries over from step to step), from
 //     alpha0 (the FP32 product of the coding pass, or, after reduced-precision
@@ -30,11 +32,13 @@
 //
 // Few signals are listed (tens to hundreds of 1e5), so the pass takes as long as
 // one signal's chain of FP64 latencies, while the rest of the GPU waits.  One
-// warp per signal with triangular solves (a division and a dependent sum per
-// selected atom and step) took 209 us at p = 64, n = 1024, s = 10 and 243 us at
-// p = 100, n = 512, s = 12.  The inverse factor turns the solves into one entry
-// per lane, eight lanes per dot product take all of a step's Gram entries (or
-// candidates) at once, and four warps share the correlations: 53 and 66 us.
+// warp per signal, with a division and a sum over shared memory for every entry of the
+// solves, took 209 us at p = 64, n = 1024, s = 10 and 243 us at p = 100, n = 512,
+// s = 12.  Here the rows of L are kept divided by their diagonal, so that an entry of
+// a solve costs a shuffle and one multiply-add, with the sums on as many lanes as there
+// are entries left; eight lanes per dot product take all of a step's Gram entries (or
+// candidates) at once, and four warps share the correlations: 55 and 72 us
+// (53 and 66 with the inverse factor).
 #include "dl_internal.cuh"
 
 #include <math.h>
@@ -68,11 +72,12 @@ __global__ void __launch_bounds__(RS_THREADS) resolve_kernel(
     const float* __restrict__ A0, int64_t lda, int n, int s, const int* __restrict__ list,
     const int* __restrict__ count, int cap, int32_t* __restrict__ oidx, float* __restrict__ oval,
     int32_t* __restrict__ ocnt) {
-  __shared__ double B[DL_RESOLVE_SMAX][DL_RESOLVE_SMAX + 1];  // L^-1, lower triangle
-  __shared__ double gd[DL_RESOLVE_SMAX + 1];                  // d_q^T d_sel, q <= k; [k + 1]: d_sel^T r
+  __shared__ double Lr[DL_RESOLVE_SMAX][DL_RESOLVE_SMAX + 1];  // L_qt / L_qq, t < q
+  __shared__ double Lc[DL_RESOLVE_SMAX][DL_RESOLVE_SMAX + 1];  // L_qt / L_tt, t < q
+  __shared__ double gd[DL_RESOLVE_SMAX + 2];                   // d_q^T d_sel, q <= k; then d_sel^T r, d_sel^T y
   __shared__ double Ds[DL_RESOLVE_SMAX][RS_PITCH];            // selected atoms
-  __shared__ double ws[DL_RESOLVE_SMAX], Gm[DL_RESOLVE_SMAX]; // new row of L; gamma
-  __shared__ double rs[RS_PMAX];                              // residual
+  __shared__ double Gm[DL_RESOLVE_SMAX];                      // gamma
+  __shared__ double rs[RS_PMAX], yd[RS_PMAX];                 // residual; y
   __shared__ double gv[RS_GROUPS], wred[RS_THREADS / 32];
   __shared__ double sh_rr, sh_gsum;
   __shared__ float ys[RS_PMAX], g32[DL_RESOLVE_SMAX];
@@ -108,7 +113,7 @@ __global__ void __launch_bounds__(RS_THREADS) resolve_kernel(
     const float yt = tid < p ? Y[i * p + tid] : 0.f;
     if (tid < p) {
       ys[tid] = yt;
-      rs[tid] = (double)yt;
+      rs[tid] = yd[tid] = (double)yt;
     }
     {
       const double t = warp_sum_d((double)yt * (double)yt);
@@ -136,6 +141,7 @@ __global__ void __launch_bounds__(RS_THREADS) resolve_kernel(
     const double ynorm = sqrt(yy);
     double rr = yy;
     double gsum = 0.0;  // sum |gamma_q|
+    double linv = 0.0, z = 0.0;  // warp 0, lane q: 1 / L_qq, z_q
     int k = 0;
     for (int step = 0; step < s; ++step) {
       if (tid == 0) ncand = 0;
@@ -212,9 +218,9 @@ __global__ void __launch_bounds__(RS_THREADS) resolve_kernel(
         if (tid + RS_THREADS * t < n)
           Gs[(size_t)k * n + tid + RS_THREADS * t] = __ldg(G + (size_t)sel * n + tid + RS_THREADS * t);
       __syncthreads();
-      // ---- FP64 Gram entries of the new atom, and d_sel^T r
-      for (int q = grp; q <= k + 1; q += RS_GROUPS) {
-        const double* x = q <= k ? Ds[q] : rs;
+      // ---- FP64 Gram entries of the new atom, d_sel^T r and d_sel^T y
+      for (int q = grp; q <= k + 2; q += RS_GROUPS) {
+        const double* x = q <= k ? Ds[q] : q == k + 1 ? rs : yd;
         double v = 0.0, v2 = 0.0;
 #pragma unroll 4
         for (int r = l8; r < p; r += 16) {
@@ -225,29 +231,34 @@ __global__ void __launch_bounds__(RS_THREADS) resolve_kernel(
         if (l8 == 0) gd[q] = v;
       }
       __syncthreads();
-      const double asel = gd[k + 1];
-      if (!(fabs(asel) > 0.0)) break;
-      // ---- Cholesky row w = B g, delta = G[sel, sel] - w.w, the new row of B, gamma += z B_k
+      if (!(fabs(gd[k + 1]) > 0.0)) break;
+      // ---- L w = g, delta = G[sel, sel] - w.w, z_k, L^T gamma = z
       if (warp == 0) {
-        double w = 0.0;
-        if (lane < k)
-          for (int t = 0; t <= lane; ++t) w = fma(B[lane][t], gd[t], w);
-        if (lane < k) ws[lane] = w;
+        double w = lane < k ? gd[lane] * linv : 0.0;
+        for (int q = 0; q + 1 < k; ++q) {
+          const double wq = __shfl_sync(FULL, w, q);
+          if (lane > q && lane < k) w = fma(-Lr[lane][q], wq, w);
+        }
         const double delta = gd[k] - warp_sum_d(w * w);
+        const double zw = gd[k + 2] - warp_sum_d(w * z);
         const bool stop = delta <= 1e-12;
         if (!stop) {
-          const double inv = rsqrt(delta), zk = asel * inv;
-          __syncwarp();
-          double b = lane == k ? inv : 0.0;
+          const double inv = rsqrt(delta), zk = zw * inv;
           if (lane < k) {
-            double acc = 0.0;
-            for (int q = lane; q < k; ++q) acc = fma(ws[q], B[q][lane], acc);
-            b = -acc * inv;
+            Lr[k][lane] = w * inv;
+            Lc[k][lane] = w * linv;
           }
-          double gm = 0.0;
+          if (lane == k) {
+            linv = inv;
+            z = zk;
+          }
+          __syncwarp();
+          double gm = z * linv;  // (zero past lane k)
+          for (int q = k; q > 0; --q) {
+            const double gq = __shfl_sync(FULL, gm, q);
+            if (lane < q) gm = fma(-Lc[q][lane], gq, gm);
+          }
           if (lane <= k) {
-            B[k][lane] = b;
-            gm = lane < k ? fma(zk, b, Gm[lane]) : zk * b;
             Gm[lane] = gm;
             g32[lane] = (float)gm;
           }
