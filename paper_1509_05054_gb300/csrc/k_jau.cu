@@ -35,23 +35,32 @@ __device__ __forceinline__ float warp_sum(float v) {
   return v;
 }
 
-// Block-wide sum of the threads' FP32 partial sums; result valid on thread 0.  FP64
-// instructions run at 1/64 of the FP32 rate, and a kernel's last CTAs all sum at
-// once (two FP64 sums of every thread cost the errors pass 3.5 us of 16.5), so the
-// warps sum unevaluated FP32 pairs (Knuth's two-sum keeps each addition's rounding
-// error, about 48 bits in all) and only one pair per warp becomes FP64.
+// Sum of the warp's 32 non-negative FP32 values in FP64: integers in units of 2^-56
+// of the largest value's binade (24 bits and 33 more), added exactly by three integer
+// reductions of 27, 27 and 3 bits each.  What is cut off and the conversion are below
+// 2^-51 of the sum, as the roundings of five FP64 additions are, over the whole range.
+__device__ __forceinline__ double warp_sum_fixed(float v) {
+  const unsigned b = __float_as_uint(v) & 0x7fffffffu;
+  const int top = (int)(__reduce_max_sync(FULL, b) >> 23);
+  if (top == 255) return (double)warp_sum(v);  // infinite or NaN, as the plain sum
+  const int ex = (int)(b >> 23), e = ex > 0 ? ex : 1, et = top > 0 ? top : 1;  // (subnormals: no leading one)
+  const unsigned long long mant = (unsigned long long)((b & 0x7fffffu) | (ex > 0 ? 0x800000u : 0u)) << 33;
+  const unsigned long long q = et - e < 57 ? mant >> (et - e) : 0ull;
+  const unsigned long long s0 = __reduce_add_sync(FULL, (unsigned)q & 0x7ffffffu);
+  const unsigned long long s1 = __reduce_add_sync(FULL, (unsigned)(q >> 27) & 0x7ffffffu);
+  const unsigned long long s2 = __reduce_add_sync(FULL, (unsigned)(q >> 54));
+  return (double)(s0 + (s1 << 27) + (s2 << 54)) * __hiloint2double((et + 840) << 20, 0);  // 2^(et - 183)
+}
+
+// Block-wide sum of the threads' FP32 partial sums (not negative); result valid on
+// thread 0.  FP64 instructions run at 1/64 of the FP32 rate, and a kernel's last CTAs
+// all sum at once (two FP64 sums of every thread cost the errors pass 3.5 us of
+// 16.5), so a warp's sum is taken in integers and only one value per warp is FP64.
 __device__ double block_sum_f(float v, double* scratch) {
   const int lane = threadIdx.x & 31, w = threadIdx.x >> 5, nw = blockDim.x >> 5;
-  float hi = v, lo = 0.f;
-#pragma unroll
-  for (int o = 16; o > 0; o >>= 1) {
-    const float oh = __shfl_xor_sync(FULL, hi, o), ol = __shfl_xor_sync(FULL, lo, o);
-    const float s = __fadd_rn(hi, oh), b = __fsub_rn(s, hi);
-    lo = __fadd_rn(__fadd_rn(lo, ol), __fadd_rn(__fsub_rn(hi, __fsub_rn(s, b)), __fsub_rn(oh, b)));
-    hi = s;
-  }
+  const double s = warp_sum_fixed(v);
   __syncthreads();
-  if (lane == 0) scratch[w] = isfinite(hi) ? (double)hi + (double)lo : (double)hi;
+  if (lane == 0) scratch[w] = s;
   __syncthreads();
   double r = 0.0;
   if (threadIdx.x == 0)
