@@ -13,7 +13,7 @@
 //      shared memory); a signal whose Cholesky pivot falls below 1e-6 is redone by
 //      the warp in FP64 with the oracle's stop rules.  (With a warp per signal, and
 //      the energies summed in FP64 signal by signal, one iteration of 200 problems
-//      at p = 20, n = 50, m = 1500, s = 4 took 616 us among others like it, now 333);
+//      at p = 20, n = 50, m = 1500, s = 4 took 616 us among others like it, now 339);
 //   3. e_i = y_i - D x_i, U = E X^T and r_j = ||x_j||^2 by shared-memory
 //      reductions (X_prev for P-NSGK, Eq. 7), ||E||^2 and ||Y||^2;
 //   4. the atom update (Eq. 5): d_j' = (U_j + r_j d_j) / ||.||, c_j = d_j^T d_j';
@@ -25,6 +25,7 @@
 #include "dl_internal.cuh"
 #include "omp_common.cuh"
 #include "omp_sub.cuh"
+#include "sum2.cuh"
 
 #include <math.h>
 
@@ -44,20 +45,6 @@ struct GramShared {
   const float* G;
   __device__ __forceinline__ float diag(int j) const { return G[j * SM_NP + j]; }
   __device__ __forceinline__ float4 vec(int row, int j) const { return *(const float4*)(G + row * SM_NP + j); }
-};
-
-// A sum of FP32 values as an unevaluated pair (Knuth's two-sum: every addition's
-// rounding error goes to lo): FP64 additions run at 1/64 of the FP32 rate.
-struct Sum2 {
-  float hi = 0.f, lo = 0.f;
-  __device__ __forceinline__ void add(float x) {
-    const float s = __fadd_rn(hi, x), b = __fsub_rn(s, hi);
-    lo = __fadd_rn(lo, __fadd_rn(__fsub_rn(hi, __fsub_rn(s, b)), __fsub_rn(x, b)));
-    hi = s;
-  }
-  __device__ __forceinline__ double value() const {
-    return isfinite(hi) ? (double)hi + (double)lo : (double)hi;
-  }
 };
 
 __device__ __forceinline__ double warp_sum_d(double v) {

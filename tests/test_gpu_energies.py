@@ -67,3 +67,19 @@ def test_energies_of_an_update_sum_past_fp32(dl, p, n, m, det):
                   torch.from_numpy(idx.astype(np.int32)).cuda(), v, rm)
     dl.dl_destroy(ctx)
     _check(rm, Dd.cpu().numpy(), p, rows)
+
+
+def test_energies_of_a_small_problem_sum_past_fp32(dl):
+    p, n, m, s = 16, 40, 128, 1
+    rows = (0, 32, 64, 96)  # (one warp, so one lane holds the axis of all four)
+    Y, D = _problem(p, n, m, rows)
+    st = torch.cuda.Stream()
+    q = dict(p=p, n=n, s=s, m=m, Y=torch.from_numpy(Y).cuda(), D=torch.from_numpy(D.copy()).cuda(),
+             colptr=torch.zeros(m + 1, dtype=torch.int64, device="cuda"),
+             rowidx=torch.zeros(m * s, dtype=torch.int32, device="cuda"), val=torch.zeros(m * s, device="cuda"))
+    torch.cuda.synchronize()
+    b = dl.dl_batch_create([q], autotune=False, stream=st)
+    rm = np.zeros(2)
+    dl.dl_batch_iterate(b, 1, rm)
+    dl.dl_batch_destroy(b)
+    _check(rm, q["D"].cpu().numpy(), p, rows)
