@@ -18,6 +18,7 @@
 // the split sums, and a layer's two backward products in one launch.  What is left is
 // mostly each launch's chain of load, MMA and epilogue latencies (about 10 us).
 #include "dl_internal.cuh"
+#include "sum2.cuh"
 #include "tc_ptx.cuh"
 
 #include <cuda.h>
@@ -75,17 +76,6 @@ __device__ __forceinline__ void load_tile(uint8_t* dst, const CUtensorMap* map, 
     tma_load_2d(dst, map, bar, k0, mn0);
   }
 }
-
-// Sum of FP32 values kept as an unevaluated pair (Knuth's two-sum: the rounding
-// error of every addition goes to lo), so that FP64 is needed once per thread.
-struct Sum2 {
-  float hi = 0.f, lo = 0.f;
-  __device__ __forceinline__ void add(float x) {
-    const float s = __fadd_rn(hi, x), b = __fsub_rn(s, hi);
-    lo += __fadd_rn(__fsub_rn(hi, __fsub_rn(s, b)), __fsub_rn(x, b));
-    hi = s;
-  }
-};
 
 __device__ __forceinline__ uint2 pack_bf16x4(float4 v) {
   const __nv_bfloat162 a = __floats2bfloat162_rn(v.x, v.y), b = __floats2bfloat162_rn(v.z, v.w);
@@ -292,7 +282,7 @@ __device__ __forceinline__ void gemm_tile(const Job& job, int bx, int by, int bz
                      "f"(cs.y), "f"(cs.z), "f"(cs.w)
                      : "memory");
     }
-    if (OP == MLP_EPI_BCE) loss = (double)ls.hi + (double)ls.lo;
+    if (OP == MLP_EPI_BCE) loss = ls.value();
   }
   if (OP == MLP_EPI_BCE) {
 #pragma unroll
