@@ -335,8 +335,10 @@ int dl_uses_tensor_cores(dl_ctx* ctx);
  * tensor-core or CUDA-core correlations, OMP warps per CTA (4/2/1), CTAs of the
  * error-accumulation pass (1x/2x), CTAs per SM of the row update (4/2/8), by a
  * coordinate search timing one DL iteration per candidate (best of 3, CUDA
- * events) from a scratch copy of D.  Y and D are device pointers and are not
- * modified.  Allocates and frees temporary device buffers and synchronises.
+ * events) from a scratch copy of D.  Only the shapes that the problem's kernels
+ * read are searched (the coding kernels other than one warp per signal and the
+ * atom update from 32 signals per SM on have fixed ones); the others keep their
+ * values.  Y and D are device pointers and are not modified.  Allocates and frees temporary device buffers and synchronises.
  * Later calls on the context use the chosen shapes.  Returns DL_OK, DL_EINVAL,
  * DL_ENOMEM or DL_ECUDA.
  */

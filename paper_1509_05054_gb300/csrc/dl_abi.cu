@@ -146,6 +146,9 @@ struct dl_ctx {
   int cfg_acc_mult = 1;   // accumulation CTAs: 1x or 2x the base count
   int cfg_row_per_sm = 4; // row-update CTAs per SM
   int cfg_corr_tc = 1;    // tensor-core correlations when the shape allows
+  // which of the four the enqueued kernels depended on since it was last cleared (bits in
+  // the order of dl_get_config): dl_autotune leaves the others alone
+  unsigned cfg_read = 0;
   // side stream: the colptr scan overlaps the first pass of the atom update
   cudaStream_t st2 = nullptr;
   cudaEvent_t ev_fork = nullptr, ev_join = nullptr, ev_join2 = nullptr;
@@ -300,9 +303,11 @@ void mark(dl_ctx* c, int k) {
 // The tensor-core path needs p % 4 == 0, p <= 64, n <= 1024 and 16-byte aligned operands;
 // other shapes use the FP32 CUDA-core GEMM.
 bool tc_ok(dl_ctx* c, const float* Y, const float* D) {
-  if (getenv("DL_FORCE_SIMT_GEMM") || !c->cfg_corr_tc) return false;
-  return dlk::corr_tc_supported(Y, c->p, c->n, c->lda) &&
-         dlk::corr_tc_supported(D, c->p, c->n, c->n);
+  if (getenv("DL_FORCE_SIMT_GEMM") || !dlk::corr_tc_supported(Y, c->p, c->n, c->lda) ||
+      !dlk::corr_tc_supported(D, c->p, c->n, c->n))
+    return false;
+  c->cfg_read |= 1u;
+  return c->cfg_corr_tc != 0;
 }
 
 cudaError_t enq_gram(dl_ctx* c, const float* D, bool tc, int* zero = nullptr) {
@@ -442,6 +447,7 @@ cudaError_t enq_batch_omp(dl_ctx* c, const float* A, bool bf16, const float* Y, 
   if (c->cfg_omp_tm && dlk::omp_sub_supported(c->n, s, m))
     return dlk::omp_sub(A, c->lda, c->G, c->n, Y, c->p, m, s, idx, val, cnt, ores, c->err, c->rs_list,
                         c->rs_count, cap, c->st);
+  c->cfg_read |= 2u;
   return dlk::omp_batch(A, c->lda, c->G, c->n, Y, c->p, m, s, idx, val, cnt, c->err, c->rs_list,
                         c->rs_count, cap, c->cfg_omp_warps, ores, gap_tol, c->st);
 }
@@ -503,6 +509,7 @@ cudaError_t enq_jau(dl_ctx* c, const float* Y, int64_t m, float* D, int s, const
                    : c->jw.E ? dlk::jau_plain_blocks(c->p)
                              : dlk::jau_accum_blocks(c->p, c->n, c->cfg_acc_mult);
   c->jw.nb_row = c->jw.E ? dlk::jau_plain_row_blocks(c->p) : dlk::jau_row_blocks(c->cfg_row_per_sm);
+  if (!c->jw.E) c->cfg_read |= c->jw.det ? 8u : 4u | 8u;
   const int nt = group_size(c);
   const int ngroups = (c->n + nt - 1) / nt;
   const bool nsgk = c->rule == DL_RULE_NSGK;
@@ -1323,15 +1330,17 @@ extern "C" int dl_autotune(dl_ctx* c, const float* Y, int64_t m, const float* D,
   c->prof = false;
   int* knobs[4] = {&c->cfg_corr_tc, &c->cfg_omp_warps, &c->cfg_acc_mult, &c->cfg_row_per_sm};
   const int choices[4][3] = {{1, 0, -1}, {4, 2, 1}, {1, 2, -1}, {4, 2, 8}};
+  c->cfg_read = 0;
   time_iteration(c, Y, m, D, Dtmp, s, cp, ri, v, e0, e1);  // warm-up
+  const unsigned read = c->cfg_read;
   float best = time_iteration(c, Y, m, D, Dtmp, s, cp, ri, v, e0, e1);
   for (int k = 0; k < 4 && rc == DL_OK; ++k) {
+    if (!(read >> k & 1u)) continue;  // every choice would time the same kernels
     const int keep = *knobs[k];
     int arg = keep;
     for (int q = 0; q < 3; ++q) {
       const int cand = choices[k][q];
       if (cand < 0 || cand == keep) continue;
-      if (k == 0 && !dlk::corr_tc_supported(Y, c->p, c->n, c->lda)) continue;
       *knobs[k] = cand;
       const float t = time_iteration(c, Y, m, D, Dtmp, s, cp, ri, v, e0, e1);
       if (t < best) {
