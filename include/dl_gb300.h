@@ -85,7 +85,10 @@ typedef struct dl_ctx dl_ctx;
  *   p          1 <= p <= DL_MAX_P.
  *   n          1 <= n <= DL_MAX_N.
  *   m_max      1 <= m_max; workspace is sized for m_max signals
- *              (about m_max * (4 max(n, p) + 8 s_max + 16) bytes plus O(n^2 + 152 n p)).
+ *              (about m_max * (4 max(n, p) + 8 s_max + 16) bytes with n rounded up to
+ *              32, 4 n^2 and 4 n (p + 1) (R + 24): R partial sums of the atom update,
+ *              two per SM, or more where the fixed summation order needs them -- a
+ *              range of signals has at most 200 KB of samples, atoms and coefficients).
  *   s_max      1 <= s_max <= min(p, n, DL_MAX_S).
  *   precision  DL_FP32, DL_BF16 or DL_FP8: the arithmetic of the correlations
  *              D^T Y (mixed precision: BF16, or E4M3 with each atom and each

@@ -876,11 +876,10 @@ int dl_init(dl_ctx** out, int p, int n, int64_t m_max, int s_max, int precision,
   if (nbd > c->jw.nb_accum) c->jw.nb_accum = (int)nbd;
   c->jw.nb_row = dlk::jau_row_blocks_max();
   const size_t ulen = dlk::jau_ulen(p, n);
-  size_t nslices = dlk::jau_accum_smem(p, n) > 0 ? (size_t)c->jw.nb_accum : 1;
-  if (nslices < (size_t)nbd) nslices = (size_t)nbd;
+  const size_t nslices = dlk::jau_slices(m_max, p, n, s_max);
   bool ok = dalloc(&c->G, (size_t)n * n) && dalloc(&c->A0, mm * std::max<int64_t>(c->lda, dlk::jau_p4(p))) &&
             dalloc(&c->sidx, mm * s_max) && dalloc(&c->sval, mm * s_max) &&
-            dalloc(&c->scnt, mm) && dalloc(&c->bsum, (size_t)2048) &&
+            dalloc(&c->scnt, mm) && dalloc(&c->bsum, (size_t)dlk::kCscBlocks) &&
             dalloc(&c->err, 1) && dalloc(&c->iter, 1) && dalloc(&c->jw.Upart, nslices * ulen) &&
             dalloc(&c->jw.U, ulen) && dalloc(&c->jw.Ucopy, dlk::jau_ulen(dlk::jau_p4(p), n) * dlk::kUCopies) && dalloc(&c->jw.epart_a, (size_t)2 * std::max(c->jw.nb_accum, dlk::jau_plain_blocks(p))) &&
             dalloc(&c->jw.epart_b, (size_t)c->jw.nb_row) && dalloc(&c->jw.Dn, (size_t)n * dlk::jau_p4(p)) &&

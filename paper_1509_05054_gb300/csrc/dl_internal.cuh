@@ -254,6 +254,10 @@ int jau_row_blocks(int per_sm);
 int jau_row_blocks_max();
 size_t jau_accum_smem(int p, int n);
 // float4 passes (p % 4 == 0, Y and D 16-byte aligned); kernel launches of the JAU passes.
+// Slices of the partial buffer Upart for up to m signals: one per range of signals in the
+// fixed summation order (p % 4 == 0; operands off 16 bytes take one), one per CTA of the
+// shared-memory form (other p), one where U itself is added to.
+size_t jau_slices(int64_t m, int p, int n, int s);
 bool jau_vec4(int p, const float* Y, const float* D);
 // Pass A with a fixed summation order, bitwise reproducible (float4 rows, p <= 128,
 // n <= 1024, s <= 16, a range of signals per CTA in shared memory); its CTA count.
@@ -279,7 +283,7 @@ cudaError_t jau_finalize(const JauWork& w, double* rmse_out, int* iter, float* D
                          cudaStream_t st);
 
 // ---- CSC <-> slots --------------------------------------------------------------
-int64_t scan_blocks(int64_t m);  // values of bsum (at most 2048)
+constexpr int kCscBlocks = 2048;  // CTAs of the scan at the most, and values of bsum: each reads all before its own
 // colptr and, when rowidx is given, the entries (values when cval is given too).
 cudaError_t slots_to_csc(const int32_t* idx, const float* val, const int32_t* cnt, int64_t m, int s,
                          int64_t* bsum, int64_t* colptr, int32_t* rowidx, float* cval, cudaStream_t st);

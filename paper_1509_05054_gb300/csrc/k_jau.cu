@@ -1357,8 +1357,10 @@ __global__ void __launch_bounds__(FIN_THREADS) finalize_kernel(
 // block sums, a serial sum over the earlier CTAs and a separate entry kernel took
 // 4.5 + 4.5 + 2.7 us at m = 60,000, s = 4; 1.9 + 4.3 us.)
 constexpr int CSC_THREADS = 256;
-constexpr int CSC_MAX_BLOCKS = 2048;  // (a CTA reads all the sums before its own)
-int csc_rounds(int64_t m) { return (int)((m + (int64_t)CSC_THREADS * CSC_MAX_BLOCKS - 1) / ((int64_t)CSC_THREADS * CSC_MAX_BLOCKS)); }
+int csc_rounds(int64_t m) {
+  const int64_t most = (int64_t)CSC_THREADS * kCscBlocks;
+  return (int)((m + most - 1) / most);
+}
 
 __global__ void __launch_bounds__(CSC_THREADS) count_sum_kernel(const int32_t* __restrict__ cnt, int64_t m,
                                                                 int rounds, int64_t* __restrict__ bsum) {
@@ -1528,6 +1530,10 @@ int jau_accum_blocks(int p, int n, int mult) {
 }
 int jau_accum_blocks_max(int p, int n) {
   return (p % 4 != 0 && jau_accum_smem(p, n) > 0) ? 2 * num_sms() : 8 * num_sms();
+}
+size_t jau_slices(int64_t m, int p, int n, int s) {
+  if (p % 4 != 0) return jau_accum_smem(p, n) > 0 ? 2 * (size_t)num_sms() : 1;
+  return jau_det_supported(p, n, s, nullptr, nullptr) ? (size_t)jau_det_ranges(m, p, n, s) : 1;
 }
 bool jau_vec4(int p, const float* Y, const float* D) {
   return p % 4 == 0 && ((uintptr_t)Y % 16) == 0 && ((uintptr_t)D % 16) == 0;
@@ -1782,16 +1788,12 @@ cudaError_t jau_finalize(const JauWork& w, double* rmse_out, int* iter, float* D
   return cudaGetLastError();
 }
 
-int64_t scan_blocks(int64_t m) {
-  const int64_t per = (int64_t)csc_rounds(m) * CSC_THREADS;
-  return per > 0 ? (m + per - 1) / per : 0;
-}
-
 cudaError_t slots_to_csc(const int32_t* idx, const float* val, const int32_t* cnt, int64_t m, int s,
                          int64_t* bsum, int64_t* colptr, int32_t* rowidx, float* cval, cudaStream_t st) {
   if (m <= 0) return cudaMemsetAsync(colptr, 0, sizeof(int64_t), st);
-  const unsigned nb = (unsigned)scan_blocks(m);
   const int rounds = csc_rounds(m);
+  const int64_t per = (int64_t)rounds * CSC_THREADS;
+  const unsigned nb = (unsigned)((m + per - 1) / per);
   count_sum_kernel<<<nb, CSC_THREADS, 0, st>>>(cnt, m, rounds, bsum);
   csc_write_kernel<<<nb, CSC_THREADS, 0, st>>>(cnt, idx, val, m, s, rounds, bsum, colptr, rowidx, cval);
   return cudaGetLastError();
