@@ -267,6 +267,12 @@ int finish(dl_ctx* c, double* rmse, int iters) {
 int ensure_rmse(dl_ctx* c, int iters) {
   if (iters <= c->rmse_cap) return DL_OK;
   DL_CHECK(cudaStreamSynchronize(c->st));
+  // captured iterations write to the array that is freed here
+  for (cudaGraphExec_t* g : {&c->gexec, &c->gexec_learned, &c->hgexec}) {
+    if (*g) cudaGraphExecDestroy(*g);
+    *g = nullptr;
+  }
+  c->gkey_seen = c->gkey_seen_l = c->hseen = 0;
   if (c->rmse) cudaFree(c->rmse);
   c->rmse = nullptr;
   c->rmse_cap = 0;
