@@ -6,12 +6,14 @@
 
 #include <cuda_bf16.h>
 #include <cuda_runtime.h>
+#include <stddef.h>
 #include <stdint.h>
 #include <stdio.h>
 #include <stdlib.h>
 #include <string.h>
 
 #include <algorithm>
+#include <type_traits>
 #include <vector>
 
 // The learned support proposer (MLP p -> hidden -> hidden -> n, BF16 weights
@@ -56,6 +58,7 @@ struct dl_ctx {
   cudaStream_t st = nullptr;
   int64_t lda = 0;  // row stride of the correlation matrix A0 (floats)
   // workspace
+  void* fixed = nullptr;  // one allocation for the arrays whose length does not depend on m_max
   float* G = nullptr;
   float* A0 = nullptr;   // m_max x max(lda, padded p): alpha0, then the errors of the atom update
   int jau_kernels = 5;   // kernel launches of the last enqueued JAU update
@@ -102,16 +105,16 @@ struct dl_ctx {
   int64_t* bsum = nullptr;
   int* err = nullptr;
   int* iter = nullptr;
-  double* rmse = nullptr;
-  int rmse_cap = 0;  // iterations
-  // page-locked landing place of the error word and of the RMSE pairs of short calls:
-  // a copy into pageable memory waits for the GPU by itself, so a call that reads
-  // both would wait twice
-  struct Landing {
+  double* rmse = nullptr;       // res->rmse, or rmse_long
+  double* rmse_long = nullptr;  // for more iterations
+  int rmse_cap = 0;             // iterations
+  // the error word and the RMSE pairs of calls of up to 64 iterations side by side: a call
+  // that reads both copies and waits once
+  struct Results {
     int err;
     double rmse[2 * 64];
   };
-  Landing* land = nullptr;
+  Results* res = nullptr;
   dlk::JauWork jw{};
   // host staging (lazily allocated)
   float* hY = nullptr;
@@ -186,14 +189,11 @@ void free_ctx(dl_ctx* c) {
   if (c->ev_join) cudaEventDestroy(c->ev_join);
   if (c->ev_join2) cudaEventDestroy(c->ev_join2);
   if (c->st2) cudaStreamDestroy(c->st2);
-  void* ptrs[] = {c->G, c->A0, c->Dhi, c->Dlo, c->Ylp, c->Ysc, c->Dlp, c->Dsc, c->rs_list,
-                  c->rs_count, c->sidx, c->sval, c->scnt, c->bsum, c->err, c->iter, c->rmse,
-                  c->jw.Upart, c->jw.U, c->jw.Ucopy, c->jw.epart_a, c->jw.epart_b, c->jw.Dn, c->jw.Dp, c->jw.C,
-                  c->hY, c->hD, c->hcolptr, c->hrowidx, c->hval, c->pidx, c->pval, c->pcnt,
+  void* ptrs[] = {c->fixed, c->A0, c->Ylp, c->Ysc, c->Dlp, c->Dsc, c->rs_list, c->sidx, c->sval, c->scnt,
+                  c->rmse_long, c->jw.Upart, c->hY, c->hD, c->hcolptr, c->hrowidx, c->hval, c->pidx, c->pval, c->pcnt,
                   c->pvalid, c->D0};
   for (void* q : ptrs)
     if (q) cudaFree(q);
-  if (c->land) cudaFreeHost(c->land);
   cudaSetDevice(prev);
   delete c;
 }
@@ -240,45 +240,41 @@ int ptr_kind(const void* p) {
   return (a.type == cudaMemoryTypeDevice || a.type == cudaMemoryTypeManaged) ? 1 : 0;
 }
 
-// Read and clear the device error word; returns a status.
-int take_device_error(dl_ctx* c) {
-  DL_CHECK(cudaMemcpyAsync(&c->land->err, c->err, sizeof(int), cudaMemcpyDeviceToHost, c->st));
+// Wait for the stream, read and clear the device error word; returns a status.  With
+// rmse the RMSE pairs of `iters` iterations too.
+int take_results(dl_ctx* c, double* rmse, int iters) {
+  const size_t bytes = sizeof(double) * 2 * (size_t)iters;
+  const bool beside = rmse && !c->rmse_long;
+  dl_ctx::Results h;
+  if (rmse && !beside) DL_CHECK(cudaMemcpyAsync(rmse, c->rmse, bytes, cudaMemcpyDeviceToHost, c->st));
+  DL_CHECK(cudaMemcpyAsync(&h, c->res, beside ? offsetof(dl_ctx::Results, rmse) + bytes : sizeof(int),
+                           cudaMemcpyDeviceToHost, c->st));
   DL_CHECK(cudaStreamSynchronize(c->st));
-  const int h = c->land->err;
-  if (h) DL_CHECK(cudaMemsetAsync(c->err, 0, sizeof(int), c->st));
-  if (h & dlk::ERR_CSC) return DL_EINVAL;
-  if (h & dlk::ERR_NONFINITE) return DL_ENUMERIC;
-  if (h & dlk::ERR_TIMEOUT) return DL_ETIMEOUT;
+  if (beside) memcpy(rmse, h.rmse, bytes);
+  if (h.err) DL_CHECK(cudaMemsetAsync(c->err, 0, sizeof(int), c->st));
+  if (h.err & dlk::ERR_CSC) return DL_EINVAL;
+  if (h.err & dlk::ERR_NONFINITE) return DL_ENUMERIC;
+  if (h.err & dlk::ERR_TIMEOUT) return DL_ETIMEOUT;
   return DL_OK;
 }
-
-// The end of a call that reads results on the host: the RMSE pairs of `iters`
-// iterations into rmse (when given) and the device error, one wait for both.
-int finish(dl_ctx* c, double* rmse, int iters) {
-  const size_t bytes = sizeof(double) * 2 * (size_t)iters;
-  const bool land = rmse && bytes <= sizeof(c->land->rmse);
-  if (rmse)
-    DL_CHECK(cudaMemcpyAsync(land ? c->land->rmse : rmse, c->rmse, bytes, cudaMemcpyDeviceToHost, c->st));
-  const int rc = take_device_error(c);
-  if (land && rc != DL_ECUDA) memcpy(rmse, c->land->rmse, bytes);
-  return rc;
-}
+int take_device_error(dl_ctx* c) { return take_results(c, nullptr, 0); }
 
 int ensure_rmse(dl_ctx* c, int iters) {
   if (iters <= c->rmse_cap) return DL_OK;
   DL_CHECK(cudaStreamSynchronize(c->st));
-  // captured iterations write to the array that is freed here
+  // captured iterations write to the array that is given up here
   for (cudaGraphExec_t* g : {&c->gexec, &c->gexec_learned, &c->hgexec}) {
     if (*g) cudaGraphExecDestroy(*g);
     *g = nullptr;
   }
   c->gkey_seen = c->gkey_seen_l = c->hseen = 0;
-  if (c->rmse) cudaFree(c->rmse);
-  c->rmse = nullptr;
-  c->rmse_cap = 0;
-  int cap = iters < 64 ? 64 : iters;
-  if (!dalloc(&c->rmse, (size_t)2 * cap)) return DL_ENOMEM;
-  c->rmse_cap = cap;
+  if (c->rmse_long) cudaFree(c->rmse_long);
+  c->rmse_long = nullptr;
+  c->rmse = c->res->rmse;
+  c->rmse_cap = 64;
+  if (!dalloc(&c->rmse_long, (size_t)2 * iters)) return DL_ENOMEM;
+  c->rmse = c->rmse_long;
+  c->rmse_cap = iters;
   return DL_OK;
 }
 
@@ -837,7 +833,7 @@ int host_call_graphed(dl_ctx* c, const float* Y, int64_t m, float* D, int s, int
     c->launches += k;
     c->hseen++;
   }
-  return finish(c, rmse, 1);
+  return take_results(c, rmse, 1);
 }
 
 }  // namespace
@@ -883,17 +879,37 @@ int dl_init(dl_ctx** out, int p, int n, int64_t m_max, int s_max, int precision,
   c->jw.nb_row = dlk::jau_row_blocks_max();
   const size_t ulen = dlk::jau_ulen(p, n);
   const size_t nslices = dlk::jau_slices(m_max, p, n, s_max);
-  bool ok = dalloc(&c->G, (size_t)n * n) && dalloc(&c->A0, mm * std::max<int64_t>(c->lda, dlk::jau_p4(p))) &&
-            dalloc(&c->sidx, mm * s_max) && dalloc(&c->sval, mm * s_max) &&
-            dalloc(&c->scnt, mm) && dalloc(&c->bsum, (size_t)dlk::kCscBlocks) &&
-            dalloc(&c->err, 1) && dalloc(&c->iter, 1) && dalloc(&c->jw.Upart, nslices * ulen) &&
-            dalloc(&c->jw.U, ulen) && dalloc(&c->jw.Ucopy, dlk::jau_ulen(dlk::jau_p4(p), n) * dlk::kUCopies) && dalloc(&c->jw.epart_a, (size_t)2 * std::max(c->jw.nb_accum, dlk::jau_plain_blocks(p))) &&
-            dalloc(&c->jw.epart_b, (size_t)c->jw.nb_row) && dalloc(&c->jw.Dn, (size_t)n * dlk::jau_p4(p)) &&
-            dalloc(&c->jw.Dp, (size_t)n * dlk::jau_p4(p)) &&
-            dalloc(&c->jw.C, (size_t)n) && dalloc(&c->Dhi, (size_t)n * p) &&
-            dalloc(&c->Dlo, (size_t)n * p) && dalloc(&c->rs_list, mm) && dalloc(&c->rs_count, 1);
-  ok = ok && cudaMallocHost((void**)&c->land, sizeof(dl_ctx::Landing)) == cudaSuccess &&
-       cudaStreamCreateWithFlags(&c->st2, cudaStreamNonBlocking) == cudaSuccess &&
+  // (an allocation takes about 10 us to make and free, a page-locked one 200)
+  const size_t p4 = (size_t)dlk::jau_p4(p);
+  size_t bytes = 0;
+  auto place = [&](auto** array, size_t count) {
+    if (c->fixed) *array = (std::remove_reference_t<decltype(*array)>)((uint8_t*)c->fixed + bytes);
+    bytes += (count * sizeof(**array) + 255) / 256 * 256;
+  };
+  auto place_all = [&] {
+    bytes = 0;
+    place(&c->G, (size_t)n * n);
+    place(&c->bsum, (size_t)dlk::kCscBlocks);
+    place(&c->res, 1);
+    place(&c->iter, 1);
+    place(&c->rs_count, 1);
+    place(&c->Dhi, (size_t)n * p);
+    place(&c->Dlo, (size_t)n * p);
+    place(&c->jw.U, ulen);
+    place(&c->jw.Ucopy, dlk::jau_ulen((int)p4, n) * dlk::kUCopies);
+    place(&c->jw.epart_a, (size_t)2 * std::max(c->jw.nb_accum, dlk::jau_plain_blocks(p)));
+    place(&c->jw.epart_b, (size_t)c->jw.nb_row);
+    place(&c->jw.Dn, n * p4);
+    place(&c->jw.Dp, n * p4);
+    place(&c->jw.C, (size_t)n);
+  };
+  place_all();  // the length
+  bool ok = dalloc((uint8_t**)&c->fixed, bytes);
+  if (ok) place_all();
+  ok = ok && dalloc(&c->A0, mm * std::max<size_t>(c->lda, p4)) && dalloc(&c->sidx, mm * s_max) &&
+       dalloc(&c->sval, mm * s_max) && dalloc(&c->scnt, mm) && dalloc(&c->rs_list, mm) &&
+       dalloc(&c->jw.Upart, nslices * ulen);
+  ok = ok && cudaStreamCreateWithFlags(&c->st2, cudaStreamNonBlocking) == cudaSuccess &&
        cudaEventCreateWithFlags(&c->ev_fork, cudaEventDisableTiming) == cudaSuccess &&
        cudaEventCreateWithFlags(&c->ev_join, cudaEventDisableTiming) == cudaSuccess &&
        cudaEventCreateWithFlags(&c->ev_join2, cudaEventDisableTiming) == cudaSuccess;
@@ -911,7 +927,10 @@ int dl_init(dl_ctx** out, int p, int n, int64_t m_max, int s_max, int precision,
     free_ctx(c);
     return DL_ENOMEM;
   }
-  if (ensure_rmse(c, 64) != DL_OK || cudaMemset(c->err, 0, sizeof(int)) != cudaSuccess ||
+  c->err = &c->res->err;
+  c->rmse = c->res->rmse;
+  c->rmse_cap = 64;
+  if (cudaMemset(c->err, 0, sizeof(int)) != cudaSuccess ||
       cudaMemset(c->iter, 0, sizeof(int)) != cudaSuccess) {
     free_ctx(c);
     return DL_ECUDA;
@@ -1144,7 +1163,7 @@ int jau_update(dl_ctx* c, const float* Y, int64_t m, float* D, const int64_t* co
     DL_CHECK(cudaMemcpyAsync(D, dD, sizeof(float) * (size_t)c->n * c->p, cudaMemcpyDeviceToHost, c->st));
     DL_CHECK(cudaMemcpyAsync(val, dv, sizeof(float) * (size_t)nnz, cudaMemcpyDeviceToHost, c->st));
   }
-  if (kind == 0 || rmse2) return finish(c, rmse2, 1);
+  if (kind == 0 || rmse2) return take_results(c, rmse2, 1);
   return DL_OK;
 }
 
@@ -1283,7 +1302,7 @@ int dl_iterate(dl_ctx* c, const float* Y, int64_t m, float* D, int s, int iters,
     DL_CHECK(cudaMemcpyAsync(rowidx, dri, sizeof(int32_t) * (size_t)m * s, cudaMemcpyDeviceToHost, c->st));
     DL_CHECK(cudaMemcpyAsync(val, dv, sizeof(float) * (size_t)m * s, cudaMemcpyDeviceToHost, c->st));
   }
-  if (kind == 0 || rmse) return finish(c, rmse, iters);
+  if (kind == 0 || rmse) return take_results(c, rmse, iters);
   return DL_OK;
 }
 
