@@ -5,7 +5,8 @@ AK-SVD atom update, group size n) on synthetic 8x8 image patches.
     python bench.py [--gpus N] [--steps K] [--warmup W] [--impl ours|reference]
 
 A step is one DL iteration over all m signals of the workload (default
-p=64, n=512, s=8, m=100000).  Prints one JSON line (rank 0).  With N > 1
+p=64, n=512, s=8, m=100000).  Prints one JSON line (rank 0) of the headline figures; the
+side measurements go to a file that it names (--details).  With N > 1
 (launched by torch.distributed.run) every rank runs an independent replica of
 the workload on its own GPU: the method needs one all-reduce of U = E X^T per
 iteration to shard one problem, which this single-GPU library does not build.
@@ -70,6 +71,8 @@ def parse():
                     help="skip timing the P-SGK and P-NSGK atom-update rules")
     ap.add_argument("--no-c1", action="store_true",
                     help="skip the p=64, n=256, s=6, m=20000 workload (50 iterations)")
+    ap.add_argument("--details", default=os.path.join(ROOT, "bench_details.json"),
+                    help="file for every measurement of the run (empty: none)")
     ap.add_argument("--m", type=int, default=None,
                     help="override the number of signals (profiling of smaller cases)")
     return ap.parse_args()
@@ -109,6 +112,25 @@ def workload_config(spec, name, extra=None):
     if extra:
         cfg.update(extra)
     return cfg
+
+
+HEADLINE = ("metric", "value", "unit", "n_gpus", "steps", "warmup", "ms_per_step", "higher_is_better",
+            "scaling", "vs_baseline", "dtype", "data", "config", "e2e", "gpu_launches", "clocks", "roofline",
+            "phases_ms")
+
+
+def headline(line, details=None):
+    """The printed line: the contract's keys, short enough for a reader that keeps the last
+    few kilobytes of the output; of the side measurements the time and RMSE of each form
+    and the CPU baseline's rate.  The whole of `line` is in the file `details`."""
+    out = {k: line[k] for k in HEADLINE}
+    out["forms"] = {f: {k: v[k] for k in ("value", "ms_per_step", "final_rmse")}
+                    for f, v in line["forms"].items()}
+    cpu = line["cpu_baseline"]
+    out["cpu_baseline"] = cpu and {k: cpu[k] for k in ("value", "unit", "cores", "kind", "sample")}
+    if details:
+        out["details"] = os.path.basename(details)
+    return out
 
 
 # ---------------------------------------------------------------- clocks
@@ -471,7 +493,10 @@ def run_ours(args):
                 "forms": forms, "atom_update_variants": variants, "batched": batched, "table1": table1,
                 "learned": learned, "c1": c1, "fp32_peak": fp32_peak,
                 "cpu_baseline": cpu, "e2e": e2e, "gpu_launches": launches, "clocks": clk}
-        print(json.dumps(line), flush=True)
+        if args.details:
+            with open(args.details, "w") as f:
+                json.dump(line, f)
+        print(json.dumps(headline(line, args.details)), flush=True)
     if pg:
         pg.destroy_process_group()
 
