@@ -12,12 +12,13 @@
 // of 4Q warps per SM keeps COLS / NT vectors of each warp's signal in TMEM
 // (256 KB per SM; warp w owns 512/Q columns of its lane quadrant, u_q[32t + l]
 // in lane l, column NT q + t) and the rest in shared memory: 16 signals per SM
-// at s <= 8, 12 at s <= 10, 8 up to s = 16 for n = 1024.  Because every vector
+// at s <= 8, 12 at s <= 10, 8 up to s = 15 and 4 at s = 16 for n = 1024.  Because every vector
 // then has an address, the loops over steps and vectors are rolled and w, c and
 // the back substitution live one entry per lane: the code is a few KB, while the
 // unrolled form with register vectors (NT (s - 1) floats per lane) is tens of KB.
-// Measured at p = 64, n = 1024, s = 10, m = 46,000: 434 us for 1,655 before;
-// what is left is the latency of each step's chain at three warps per scheduler.
+// Measured at p = 64, n = 1024, s = 10, m = 46,000: 430 us for 1,655 before, at
+// 0.54 instructions per scheduler and cycle with three warps each: about half of
+// the time is issue, the rest the latency of each step's chain.
 #include "dl_internal.cuh"
 #include "omp_common.cuh"
 #include "tc_ptx.cuh"

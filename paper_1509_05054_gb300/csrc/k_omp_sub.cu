@@ -1,6 +1,6 @@
 // Batch-OMP sparse coding of several signals per warp, for small dictionaries and
-// short supports (Algorithm 1 step 1; n <= 256, s <= 8; the arithmetic of
-// omp_warp_kernel, see k_omp.cu, operation by operation, so the results are the
+// short supports (Algorithm 1 step 1; n <= 128 and s <= 8, n <= 256 and s <= 6; the
+// arithmetic of omp_warp_kernel, see k_omp.cu, operation by operation, so the results are the
 // same bits).
 //
 // With n = 128 a warp per signal leaves each lane four correlations, and most of

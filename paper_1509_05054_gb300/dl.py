@@ -270,8 +270,9 @@ def dl_autotune(ctx: int, Y, m: int, D, s: int) -> None:
 
 
 def dl_last_omp_kernel(ctx: int) -> int:
-    """The coding kernel of the last pass: 0 Batch-OMP (warp), 1 Batch-OMP (TMEM),
-    2 residual-form tensor-core OMP, 3 restricted to proposed candidates, -1 none."""
+    """The coding kernel of the last pass: 0 Batch-OMP with one or several signals per warp,
+    1 Batch-OMP with its vectors in TMEM or, for wide dictionaries and long supports, shared
+    memory, 2 residual-form tensor-core OMP, 3 restricted to proposed candidates, -1 none."""
     out = ctypes.c_int(0)
     _check(load().dl_last_omp_kernel(ctx, ctypes.byref(out)), "dl_last_omp_kernel")
     return int(out.value)
