@@ -69,3 +69,29 @@ def test_coefficients_of_near_dependent_supports(dl, p, eps, tol, seed):
     assert same.all() if eps > 5e-5 else same.mean() > 0.8
     scale = np.abs(val_o).max(1, keepdims=True)
     assert (np.abs(val - val_o) / scale)[same].max() < tol
+
+
+@pytest.mark.parametrize("p,n,s,m", [(64, 300, 9, 2000), (49, 130, 10, 700)])
+def test_many_listed_signals_with_several_candidates_per_step(dl, p, n, s, m):
+    """Every atom has a twin within 1e-6 of it: the two correlations lie inside the FP32
+    error of each other at every step, so every signal is listed (more than there are CTAs)
+    and the re-solve tells the candidates apart in FP64, as the oracle does."""
+    g = np.random.default_rng(n)
+    A = g.standard_normal((n // 2, p))
+    D = np.vstack([A, A + 1e-6 * np.linalg.norm(A, axis=1, keepdims=True) * g.standard_normal(A.shape) / np.sqrt(p)])
+    D = (D / np.linalg.norm(D, axis=1, keepdims=True)).astype(np.float32)[g.permutation(len(D))]
+    Y = g.standard_normal((m, p)).astype(np.float32)
+    ctx = dl.dl_init(p, len(D), m, s, dl.DL_FP32, torch.cuda.current_stream())
+    cp = torch.zeros(m + 1, dtype=torch.int64, device="cuda")
+    ri = torch.zeros(m * s, dtype=torch.int32, device="cuda")
+    v = torch.zeros(m * s, device="cuda")
+    dl.omp_code(ctx, torch.from_numpy(Y).cuda(), m, torch.from_numpy(D).cuda(), s, cp, ri, v)
+    dl.dl_sync(ctx)
+    listed = dl.dl_last_resolved(ctx)
+    dl.dl_destroy(ctx)
+    assert listed == m
+    idx, val, cnt = csc_to_slots(cp.cpu().numpy(), ri.cpu().numpy(), v.cpu().numpy(), s)
+    idx_o, val_o, cnt_o = oracle.omp(Y.astype(np.float64), D.astype(np.float64), s)
+    np.testing.assert_array_equal(cnt, cnt_o)
+    np.testing.assert_array_equal(idx, idx_o)
+    np.testing.assert_allclose(val, val_o, rtol=0, atol=1e-6 * np.abs(val_o).max())
