@@ -494,8 +494,12 @@ def run_ours(args):
                 "learned": learned, "c1": c1, "fp32_peak": fp32_peak,
                 "cpu_baseline": cpu, "e2e": e2e, "gpu_launches": launches, "clocks": clk}
         if args.details:
-            with open(args.details, "w") as f:
-                json.dump(line, f)
+            try:
+                with open(args.details, "w") as f:
+                    json.dump(line, f)
+            except OSError as e:  # (the printed line does not depend on it)
+                print(f"details not written: {e}", file=sys.stderr)
+                args.details = None
         print(json.dumps(headline(line, args.details)), flush=True)
     if pg:
         pg.destroy_process_group()
